@@ -120,6 +120,106 @@ __device__ __noinline__ void rs_mask_chunk(uint32_t taddr, int mode, int i, int 
   tc_wait_st();
 }
 
+// ------------------------------------------------------------------------------------------ softmax (one row per thread)
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max32(const uint32_t (&x)[32]) {
+  float mx0 = max3(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2]));
+  float mx1 = max3(__uint_as_float(x[3]), __uint_as_float(x[4]), __uint_as_float(x[5]));
+  float mx2 = max3(__uint_as_float(x[6]), __uint_as_float(x[7]), __uint_as_float(x[8]));
+  float mx3 = max3(__uint_as_float(x[9]), __uint_as_float(x[10]), __uint_as_float(x[11]));
+#pragma unroll
+  for (int q = 12; q < 28; q += 8) {
+    mx0 = max3(mx0, __uint_as_float(x[q]), __uint_as_float(x[q + 1]));
+    mx1 = max3(mx1, __uint_as_float(x[q + 2]), __uint_as_float(x[q + 3]));
+    mx2 = max3(mx2, __uint_as_float(x[q + 4]), __uint_as_float(x[q + 5]));
+    mx3 = max3(mx3, __uint_as_float(x[q + 6]), __uint_as_float(x[q + 7]));
+  }
+  mx0 = max3(mx0, __uint_as_float(x[28]), __uint_as_float(x[29]));
+  mx1 = max3(mx1, __uint_as_float(x[30]), __uint_as_float(x[31]));
+  return fmaxf(max3(mx0, mx1, mx2), mx3);
+}
+// P = exp2(x * sl2 - m) of 32 scores as bf16 pairs; the sum of the unrounded values is returned.
+__device__ __forceinline__ float exp32(const uint32_t (&x)[32], uint32_t (&pk)[16], float sl2, float m_use) {
+  uint64_t acc = 0ull, acc_b = 0ull;     // two packed pairs of fp32 partial sums
+  uint64_t sl2x2, negm2;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(sl2x2) : "f"(sl2));
+  asm("mov.b64 %0, {%1, %1};" : "=l"(negm2) : "f"(-m_use));
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    uint64_t s2, t2, p2;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(s2) : "r"(x[2 * q]), "r"(x[2 * q + 1]));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t2) : "l"(s2), "l"(sl2x2), "l"(negm2));
+    float t0, t1;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(t2));
+    const float p0 = fast_exp2(t0), p1 = fast_exp2(t1);
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p2) : "f"(p0), "f"(p1));
+    if (q & 1) { asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc_b) : "l"(acc_b), "l"(p2)); }
+    else       { asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc) : "l"(acc), "l"(p2)); }
+    pk[q] = pack_bf16x2(p0, p1);
+  }
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc) : "l"(acc), "l"(acc_b));
+  float a0, a1;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a0), "=f"(a1) : "l"(acc));
+  return a0 + a1;
+}
+// l and O (t_o, 128 columns) of the warp's rows times alpha.  No product into O may be in flight.
+__device__ __forceinline__ void rescale(float alpha, float& l_run, bool has_o, uint32_t t_o) {
+  l_run *= alpha;
+  if (!has_o) return;
+  uint32_t w[16];
+#pragma unroll 1
+  for (uint32_t c = 0; c < 128u; c += 16u) {
+    tmem_ld16(t_o + c, w);
+    tc_wait_ld16(w);
+#pragma unroll
+    for (int q = 0; q < 16; ++q) w[q] = __float_as_uint(__uint_as_float(w[q]) * alpha);
+    tmem_st16(t_o + c, w);
+  }
+  tc_wait_st();
+}
+// Raises the running maximum of the warp's rows to m_new where that is larger.
+__device__ __forceinline__ void raise_maximum(float m_new, float& m_run, float& l_run, bool has_o, uint32_t t_o) {
+  m_new = fmaxf(m_new, m_run);
+  const float alpha = (m_new == -INFINITY) ? 1.0f : fast_exp2(m_run - m_new);
+  m_run = m_new;
+  rescale(alpha, l_run, has_o, t_o);
+}
+// The reference m of a row's exponentials need not be its maximum: any value that keeps the sums in range gives the same
+// result.  So there is no maximum pass over the scores (a fifth of the softmax instructions); the sum over the 64 keys of a
+// chunk, which is there anyway, bounds the largest of them, and m is raised to the true maximum when that sum exceeds
+// kSumBig, or while the row has no finite m yet.  At the power cap a launch is paid in instructions: dense 32K 8.05 ->
+// 7.83 ms back to back, 6.95 -> 6.78 ms singly; routed 32K 3.29 -> 3.14 ms (with the issuer's change below).
+constexpr float kSumBig = 256.0f;
+
+// The rare case, out of line: raises m to the maximum of the 64 scores at t_x, then forms their probabilities again.
+// Returns m, l (rescaled, without these 64) and the sum over them.
+__device__ __noinline__ float3 rs_raise_and_exp(uint32_t t_x, float sl2, float m_run, float l_run, bool has_o,
+                                                uint32_t t_o) {
+  uint32_t v[32], pk0[16], pk1[16];
+  float mx = -INFINITY;
+#pragma unroll 1
+  for (uint32_t c = 0; c < 64u; c += 32u) {
+    tmem_ld32(t_x + c, v);
+    tc_wait_ld32(v);
+    mx = fmaxf(mx, max32(v));
+  }
+  raise_maximum(mx * sl2, m_run, l_run, has_o, t_o);
+  const float m_use = (m_run == -INFINITY) ? 0.f : m_run;
+  tmem_ld32(t_x, v);
+  tc_wait_ld32(v);
+  float sum = exp32(v, pk0, sl2, m_use);
+  tmem_ld32(t_x + 32u, v);
+  tc_wait_ld32(v);
+  sum += exp32(v, pk1, sl2, m_use);
+  tmem_st16(t_x, pk0);
+  tmem_st16(t_x + 16u, pk1);
+  return make_float3(m_run, l_run, sum);
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
 rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKp,
@@ -129,7 +229,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sm = smem_raw + (base - raw);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
 
   // ---- work item
   const int2 w = P.order[blockIdx.x];
@@ -182,7 +282,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = (uint32_t)misc[0];
+  const uint32_t tmem = (uint32_t)warp_uniform(misc[0]);
 
   // Q tile load goes out before the chunk list is built.
   if (tid == 0) {
@@ -327,7 +427,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
   }
   __syncthreads();
-  const int n_block = misc[2], n_vert = (misc[3] + kChunk - 1) / kChunk;     // misc[3]: visible gathered columns
+  const int n_block = warp_uniform(misc[2]), n_vert = (warp_uniform(misc[3]) + kChunk - 1) / kChunk;     // misc[3]: visible gathered columns
   const int n_chunks = n_block + n_vert;
   // =========================================================================================== roles
   // Everything below is pipelined per 64-key chunk; chunk c uses slot c & 1 of the K / V rings, of the two 64-column
@@ -369,63 +469,65 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       if (!ok) { rs_report(P.status, RS_ERR_TIMEOUT, site); *abort_flag = 1; }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ MMA issuer
-      const uint32_t d_s = tmem + kColS, d_o = tmem + kColO;
-      // Descriptor words are formed once; an instruction then costs the issuing thread two adds and the MMA itself.
-      const uint64_t q_desc = umma_smem_desc(base + SmemLayout::q, 16, 1024);
-      const uint64_t k_desc = umma_smem_desc(base + SmemLayout::k, 16, 1024);
-      const uint64_t v_desc = umma_smem_desc(base + SmemLayout::v, 16384, 1024);
-      const uint32_t q_lo = (uint32_t)q_desc, q_hi = (uint32_t)(q_desc >> 32);
-      const uint32_t k_lo = (uint32_t)k_desc, k_hi = (uint32_t)(k_desc >> 32);
-      const uint32_t v_lo = (uint32_t)v_desc, v_hi = (uint32_t)(v_desc >> 32);
-      constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 64, 0, 0);
-      constexpr uint32_t kIdescPV = umma_idesc_bf16(128, 128, 0, 1);
-      auto issue_qk = [&](uint32_t slot) {      // S[slot] = Q K[slot]^T: 8 steps of 16 head dimensions
-        const uint32_t kb = k_lo + slot * 512u, ds = d_s + slot * 64u;
+    // -------------------------------------------------------------------- MMA issuer
+    // The whole warp runs the code and one elected lane issues: operands of warp-uniform code sit in uniform registers.
+    // From inside a lane == 0 branch every operand word is moved there per instruction: 16 instructions with a barrier wait
+    // between them took 1430 to 1790 clocks against 1025 of execution, and the pipe's queue never filled.
+    const bool leader = elect_one();
+    const uint32_t d_s = tmem + kColS, d_o = tmem + kColO;
+    // Descriptor words are formed once; an instruction then costs the issuing thread two adds and the MMA itself.
+    const uint64_t q_desc = umma_smem_desc(base + SmemLayout::q, 16, 1024);
+    const uint64_t k_desc = umma_smem_desc(base + SmemLayout::k, 16, 1024);
+    const uint64_t v_desc = umma_smem_desc(base + SmemLayout::v, 16384, 1024);
+    const uint32_t q_lo = (uint32_t)q_desc, q_hi = (uint32_t)(q_desc >> 32);
+    const uint32_t k_lo = (uint32_t)k_desc, k_hi = (uint32_t)(k_desc >> 32);
+    const uint32_t v_lo = (uint32_t)v_desc, v_hi = (uint32_t)(v_desc >> 32);
+    constexpr uint32_t kIdescQK = umma_idesc_bf16(128, 64, 0, 0);
+    constexpr uint32_t kIdescPV = umma_idesc_bf16(128, 128, 0, 1);
+    auto issue_qk = [&](uint32_t slot) {      // S[slot] = Q K[slot]^T: 8 steps of 16 head dimensions
+      const uint32_t kb = k_lo + slot * 512u, ds = d_s + slot * 64u;
+      if (!leader) return;
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t off = (uint32_t)(((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
-          umma_ss2(ds, q_lo + off, q_hi, kb + off, k_hi, kIdescQK, kk > 0 ? 1u : 0u);
-        }
-      };
-      auto issue_pv = [&](uint32_t slot, bool accumulate) {   // O += P[slot] V[slot]: 4 steps of 16 keys
-        const uint32_t vb = v_lo + slot * 512u, ps = d_s + slot * 64u;
-        umma_ts2(d_o, ps, vb, v_hi, kIdescPV, accumulate ? 1u : 0u);
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint32_t off = (uint32_t)(((kk >> 2) * 16384 + (kk & 3) * 32) >> 4);
+        umma_ss2(ds, q_lo + off, q_hi, kb + off, k_hi, kIdescQK, kk > 0 ? 1u : 0u);
+      }
+      umma_commit(bar_s + 8u * slot);
+      umma_commit(bar_ke + 8u * slot);
+    };
+    auto issue_pv = [&](uint32_t slot, bool accumulate) {   // O += P[slot] V[slot]: 4 steps of 16 keys
+      const uint32_t vb = v_lo + slot * 512u, ps = d_s + slot * 64u;
+      if (!leader) return;
+      umma_ts2(d_o, ps, vb, v_hi, kIdescPV, accumulate ? 1u : 0u);
 #pragma unroll
-        for (int kk = 1; kk < 4; ++kk) umma_ts2(d_o, ps + 8u * kk, vb + 128u * kk, v_hi, kIdescPV, 1u);
-      };
-      bool ok = mbar_wait(bar_q, 0, abort_flag);
-      int site = 3;
-      for (int c = 0; c < 2 && c < n_chunks && ok; ++c) {
-        ok = mbar_wait(bar_kf + 8u * c, 0, abort_flag); site = 4;
-        if (!ok) break;
-        tc_fence_after();
-        issue_qk((uint32_t)c);
-        umma_commit(bar_s + 8u * c);
-        umma_commit(bar_ke + 8u * c);
-      }
-      for (int c = 0; c < n_chunks && ok; ++c) {
-        const uint32_t slot = (uint32_t)(c & 1), ph = (uint32_t)((c >> 1) & 1);
-        ok = mbar_wait(bar_p + 8u * slot, ph, abort_flag); site = 5;
-        if (!ok) break;
-        ok = mbar_wait(bar_vf + 8u * slot, ph, abort_flag); site = 6;
-        if (!ok) break;
-        tc_fence_after();
-        issue_pv(slot, c > 0);
-        umma_commit(bar_ve + 8u * slot);
-        if (c + 2 < n_chunks) {
-          ok = mbar_wait(bar_kf + 8u * slot, ph ^ 1u, abort_flag); site = 7;
-          if (!ok) break;
-          tc_fence_after();
-          issue_qk(slot);
-          umma_commit(bar_s + 8u * slot);
-          umma_commit(bar_ke + 8u * slot);
-        }
-      }
-      if (ok) umma_commit(bar_o);
-      if (!ok) { rs_report(P.status, RS_ERR_TIMEOUT, site); *abort_flag = 1; }
+      for (int kk = 1; kk < 4; ++kk) umma_ts2(d_o, ps + 8u * kk, vb + 128u * kk, v_hi, kIdescPV, 1u);
+      umma_commit(bar_ve + 8u * slot);
+    };
+    bool ok = mbar_wait_lean(bar_q, 0, abort_flag);
+    int site = 3;
+    for (int c = 0; c < 2 && c < n_chunks && ok; ++c) {
+      ok = mbar_wait_lean(bar_kf + 8u * c, 0, abort_flag); site = 4;
+      if (!ok) break;
+      tc_fence_after();
+      issue_qk((uint32_t)c);
     }
+    for (int c = 0; c < n_chunks && ok; ++c) {
+      const uint32_t slot = (uint32_t)(c & 1), ph = (uint32_t)((c >> 1) & 1);
+      ok = mbar_wait_lean(bar_p + 8u * slot, ph, abort_flag); site = 5;
+      if (!ok) break;
+      ok = mbar_wait_lean(bar_vf + 8u * slot, ph, abort_flag); site = 6;
+      if (!ok) break;
+      tc_fence_after();
+      issue_pv(slot, c > 0);
+      if (c + 2 < n_chunks) {
+        ok = mbar_wait_lean(bar_kf + 8u * slot, ph ^ 1u, abort_flag); site = 7;
+        if (!ok) break;
+        tc_fence_after();
+        issue_qk(slot);
+      }
+    }
+    if (ok && leader) umma_commit(bar_o);
+    if (!ok && leader) { rs_report(P.status, RS_ERR_TIMEOUT, site); *abort_flag = 1; }
   } else {
     // -------------------------------------------------------------------- softmax / correction / epilogue
     const int quad = warp & 3;
@@ -440,61 +542,14 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const int* vcols = P.idx.vs_cols + (size_t)vs_slot * P.idx.kv_cap;
     bool ok = true;
     uint32_t v[32], v2[32];
-    auto max3 = [](float a, float b, float c) -> float {
-      float d;
-      asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-      return d;
-    };
-    auto max32 = [&](const uint32_t (&x)[32]) -> float {
-      float mx0 = max3(__uint_as_float(x[0]), __uint_as_float(x[1]), __uint_as_float(x[2]));
-      float mx1 = max3(__uint_as_float(x[3]), __uint_as_float(x[4]), __uint_as_float(x[5]));
-      float mx2 = max3(__uint_as_float(x[6]), __uint_as_float(x[7]), __uint_as_float(x[8]));
-      float mx3 = max3(__uint_as_float(x[9]), __uint_as_float(x[10]), __uint_as_float(x[11]));
-#pragma unroll
-      for (int q = 12; q < 28; q += 8) {
-        mx0 = max3(mx0, __uint_as_float(x[q]), __uint_as_float(x[q + 1]));
-        mx1 = max3(mx1, __uint_as_float(x[q + 2]), __uint_as_float(x[q + 3]));
-        mx2 = max3(mx2, __uint_as_float(x[q + 4]), __uint_as_float(x[q + 5]));
-        mx3 = max3(mx3, __uint_as_float(x[q + 6]), __uint_as_float(x[q + 7]));
-      }
-      mx0 = max3(mx0, __uint_as_float(x[28]), __uint_as_float(x[29]));
-      mx1 = max3(mx1, __uint_as_float(x[30]), __uint_as_float(x[31]));
-      return fmaxf(max3(mx0, mx1, mx2), mx3);
-    };
-    auto exp_chunk = [&](const uint32_t (&x)[32], uint32_t dst, float m_use) {
-      uint32_t pk[16];
-      uint64_t acc = 0ull, acc_b = 0ull;     // two packed pairs of fp32 partial sums
-      uint64_t sl2x2, negm2;
-      asm("mov.b64 %0, {%1, %1};" : "=l"(sl2x2) : "f"(sl2));
-      asm("mov.b64 %0, {%1, %1};" : "=l"(negm2) : "f"(-m_use));
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        uint64_t s2, t2, p2;
-        asm("mov.b64 %0, {%1, %2};" : "=l"(s2) : "r"(x[2 * q]), "r"(x[2 * q + 1]));
-        asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(t2) : "l"(s2), "l"(sl2x2), "l"(negm2));
-        float t0, t1;
-        asm("mov.b64 {%0, %1}, %2;" : "=f"(t0), "=f"(t1) : "l"(t2));
-        const float p0 = fast_exp2(t0), p1 = fast_exp2(t1);
-        asm("mov.b64 %0, {%1, %2};" : "=l"(p2) : "f"(p0), "f"(p1));
-        if (q & 1) { asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc_b) : "l"(acc_b), "l"(p2)); }
-        else       { asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc) : "l"(acc), "l"(p2)); }
-        pk[q] = pack_bf16x2(p0, p1);
-      }
-      asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc) : "l"(acc), "l"(acc_b));
-      float a0, a1;
-      asm("mov.b64 {%0, %1}, %2;" : "=f"(a0), "=f"(a1) : "l"(acc));
-      l_run += a0 + a1;
-      tmem_st16(dst, pk);
-    };
-
-    // One pass per 64-key chunk: rare chunks are masked in place first, then the scores go to registers (two
-    // 32-column loads per wait), chunk maximum, P = exp2(S * scale*log2e - m) against the running maximum, bf16 P
-    // over the start of the chunk's score buffer.  The maximum only moves when some row of the warp exceeds it by more
-    // than 2^8; then l and O are rescaled, after the product of the previous chunk has left the tensor pipe.
+    // One pass per 64-key chunk: rare chunks are masked in place first, then the scores go to registers,
+    // P = exp2(S * scale*log2e - m) against the row's reference m (first: the maximum of the row's first 32 scores), bf16 P
+    // over the start of the chunk's score buffer.  m is raised only when the sums say so (kSumBig); then l and O are
+    // rescaled, after the product of the previous chunk has left the tensor pipe.
     for (int ch = 0; ch < n_chunks; ++ch) {
       const uint32_t slot = (uint32_t)(ch & 1), ph = (uint32_t)((ch >> 1) & 1);
       const uint32_t t_sc = t_s + slot * 64u;
-      ok = mbar_wait(bar_s + 8u * slot, ph, abort_flag);
+      ok = mbar_wait_lean(bar_s + 8u * slot, ph, abort_flag);
       if (!ok) break;
       tc_fence_after();
       {
@@ -536,36 +591,29 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         if (mode >= 0) rs_mask_chunk(t_sc, mode, i, j0, edge, cand.b0, cand.b1, vcols, vbase, n_vcols, d_bits, vk, vd);
       }
       tmem_ld32(t_sc, v);
+      tc_wait_ld32(v);
       tmem_ld32(t_sc + 32u, v2);
-      tc_wait_ld();
-      const float m_chunk = fmaxf(max32(v), max32(v2)) * sl2;
-      const float m_new = fmaxf(m_run, m_chunk);
-      const bool need = m_new > m_run + 8.0f;
-      if (__any_sync(0xffffffffu, need)) {
-        const float alpha = (m_new == NEG_INF) ? 1.0f : fast_exp2(m_run - m_new);
-        l_run *= alpha;
-        m_run = m_new;
+      if (m_run == NEG_INF) m_run = max32(v) * sl2;
+      const float m_use = (m_run == NEG_INF) ? 0.f : m_run;
+      uint32_t pk0[16], pk1[16];
+      float sum = exp32(v, pk0, sl2, m_use);
+      tc_wait_ld32(v2);
+      sum += exp32(v2, pk1, sl2, m_use);
+      if (__any_sync(0xffffffffu, sum > kSumBig || m_run == NEG_INF)) {
         if (ch > 0) {
           // O holds the products up to chunk ch - 1; the last of them may still be in flight
           const uint32_t pslot = (uint32_t)((ch - 1) & 1), pph = (uint32_t)(((ch - 1) >> 1) & 1);
           ok = mbar_wait(bar_ve + 8u * pslot, pph, abort_flag);
           if (!ok) break;
           tc_fence_after();
-          uint32_t w32[32];
-#pragma unroll 1
-          for (int c4 = 0; c4 < 4; ++c4) {
-            tmem_ld32(t_o + (uint32_t)c4 * 32u, w32);
-            tc_wait_ld();
-#pragma unroll
-            for (int q = 0; q < 32; ++q) w32[q] = __float_as_uint(__uint_as_float(w32[q]) * alpha);
-            tmem_st32(t_o + (uint32_t)c4 * 32u, w32);
-          }
-          tc_wait_st();
         }
+        const float3 f = rs_raise_and_exp(t_sc, sl2, m_run, l_run, ch > 0, t_o);
+        m_run = f.x; l_run = f.y; sum = f.z;
+      } else {
+        tmem_st16(t_sc, pk0);
+        tmem_st16(t_sc + 16u, pk1);
       }
-      const float m_use = (m_run == NEG_INF) ? 0.f : m_run;
-      exp_chunk(v, t_sc, m_use);
-      exp_chunk(v2, t_sc + 16u, m_use);
+      l_run += sum;
       tc_wait_st();
       tc_fence_before();
       mbar_arrive(bar_p + 8u * slot);

@@ -182,3 +182,32 @@ def test_many_vertical_columns_cover_both_mask_paths():
     Oo, lo, _ = A.masked_attention(Qs[0], Ks[0], Vs[0], lambda r, nk: PT.mask_rows(ix, r, nk), rows)
     assert_attention_close(O[0].cpu().numpy()[rows], Oo, "many verticals")
     assert np.abs(lse[0].cpu().numpy()[rows] - lo).max() < 2e-3
+
+
+@pytest.mark.parametrize("steps", [
+    [0.0, 3.0, 6.0, 9.0, 12.0],            # every chunk exceeds the reference by a few powers of two: lazily, then raised
+    [0.0, 0.0, 90.0, 90.0, -90.0],         # one jump inside the range of the exponentials
+    [-180.0, -180.0, 120.0, 0.0, 180.0],   # first scores far below zero; jumps beyond the range (exp2 of them overflows)
+])
+@pytest.mark.parametrize("offset", [0, 17, 40])
+def test_dense_when_scores_climb(steps, offset):
+    """The reference of a row's exponentials is raised when the sums over a chunk grow, not by a maximum pass: scores that
+    climb from chunk to chunk, with the step at the chunk's start, inside its first and inside its second half.
+    Probabilities are rounded to bf16 relative to themselves, so the oracle's tolerance holds at every reference."""
+    n = 64 * len(steps)
+    rng = np.random.default_rng(3 + offset)
+    level = np.repeat(np.array(steps), 64)
+    level = np.concatenate([np.full(offset, level[0]), level])[:n]
+    Q, K, V = (rng.standard_normal((1, n, 128)) for _ in range(3))
+    Q[0, :, 0], K[0, :, 0] = 16.0, level * np.sqrt(128.0) * np.log(2.0) / 16.0      # level: powers of two added to the score
+    as_bf16 = lambda x: torch.from_numpy(x).to(torch.bfloat16)
+    q, k, v = as_bf16(Q), as_bf16(K), as_bf16(V)
+    p = rs.Problem(1, 1, n)
+    O = torch.zeros((1, n, 128), dtype=torch.float32, device="cuda")
+    lse, onorm, st = torch.zeros((1, n), device="cuda"), torch.zeros((1, n), device="cuda"), rs.new_status()
+    rs.rs_dense_prefill_attn(p, q.cuda(), k.cuda(), v.cuda(), O, lse, onorm, None, rs.new_workspace(p, None), st)
+    rs.check_status(st, "climbing scores")
+    Oo, lo = A.dense_attention(*(x[0].double().numpy() for x in (q, k, v)))
+    assert_attention_close(O[0].cpu().numpy(), Oo, f"steps {steps} offset {offset}")
+    # scores of magnitude 2^7 carry 2^-17 of it as fp32 rounding of the scaled product, on top of the 2e-3 of the other tests
+    assert np.abs(lse[0].cpu().numpy() - lo).max() < 2e-3 + np.abs(lo).max() * 2.0 ** -17
