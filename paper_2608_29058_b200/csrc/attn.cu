@@ -751,9 +751,21 @@ rs_attn_prepare_kernel(AttnParams P, int n_groups, int per_group, int n_bins, in
     atomicAdd(&hist[c], 1);
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int acc = 0;
-    for (int b = n_bins - 1; b >= 0; --b) { int c = hist[b]; hist[b] = acc; acc += c; }
+  if (threadIdx.x < 32) {                   // first position of every bin, heaviest bin first: warp scans of 32 bins
+    const int lane = threadIdx.x;
+    int carry = 0;
+    for (int top = n_bins - 1; top >= 0; top -= 32) {
+      const int b = top - lane;
+      const int c = b >= 0 ? hist[b] : 0;
+      int incl = c;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += t;
+      }
+      if (b >= 0) hist[b] = carry + incl - c;
+      carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < per_group; i += blockDim.x) {

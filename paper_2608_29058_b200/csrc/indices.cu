@@ -397,6 +397,233 @@ rs_vs_select_kernel(IdxParams P) {
   cluster.sync();                                        // no block leaves while its totals may still be read
 }
 
+// ------------------------------------------------------------------------------------------ the same for short lists
+// One block of 1024 threads per list, its keys in shared memory.  What bounds a selection of a few thousand keys is latency:
+// the cluster's is three cluster barriers and remote shared-memory reads per digit, here a digit costs a few block barriers,
+// and digits above the largest key are skipped.  The loops are not unrolled: the kernel runs once per layer, and a first
+// pass over its instructions costs more than their issue.  Warp w owns a contiguous range, so positions come in index order.
+constexpr int kBlkThreads = 1024, kBlkWarps = kBlkThreads / 32;
+constexpr int kBlockSelMax = 16384;
+
+__global__ void __launch_bounds__(kBlkThreads, 1)
+rs_vs_select_block_kernel(IdxParams P) {
+  extern __shared__ u64 skeys[];                          // the domain's keys
+  __shared__ unsigned int hist[kSelMaxC][kBins];
+  __shared__ unsigned int wtot[kSelMaxC][kBlkWarps], w_gt[kSelMaxC][kBlkWarps], w_eq[kSelMaxC][kBlkWarps];
+  __shared__ u64 sh_prefix[kSelMaxC], sh_max;
+  __shared__ unsigned int sh_k[kSelMaxC];
+  const int list = blockIdx.x & 1, item = blockIdx.x >> 1;
+  int cand_id[kSelMaxC] = {}, slot_id[kSelMaxC] = {}, kk[kSelMaxC] = {};
+  int nC = 0;
+  {
+    int seen = 0;
+    for (int c = 0; c < P.n_cand; ++c) {
+      if (P.lib[c].pattern != RS_VERTICAL_SLASH) continue;
+      if (P.choice != nullptr && P.choice[item] != c) continue;
+      if (seen / kSelMaxC == (int)blockIdx.y && nC < kSelMaxC) {
+        const int sl = (P.choice != nullptr) ? item : item * P.n_cand + c;
+        _Pragma("unroll") for (int e = 0; e < kSelMaxC; ++e) if (e == nC) { cand_id[e] = c; slot_id[e] = sl; }
+        ++nC;
+      }
+      ++seen;
+    }
+  }
+  if (nC == 0) return;
+  const int q1 = P.seg_bounds[item / P.Hq + 1];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u64* keys = P.keys + ((size_t)item * 2 + list) * P.n;
+  const int first = (list == 0) ? 0 : 1;                 // first index of the domain
+  const int n_dom = q1 - first;
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC) {
+    const rs_candidate cand = P.lib[cand_id[c]];
+    kk[c] = min(max((list == 0) ? min(cand.b0, q1) : (min(cand.b1, q1) - 1), 0), n_dom);
+  }
+  const int cap = (list == 0) ? P.out.kv_cap : P.out.ks_cap;
+  const int chunk = ((n_dom + kBlkThreads - 1) / kBlkThreads) * 32;
+  const int lo = min(n_dom, warp * chunk), hi = min(n_dom, lo + chunk);
+  if (tid == 0) sh_max = 0;
+  if (tid < kSelMaxC) { sh_prefix[tid] = 0; }
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (tid == c) sh_k[c] = c < nC ? (unsigned)kk[c] : 0u;
+  __syncthreads();
+  {
+    u64 mx = 0;
+#pragma unroll 4
+    for (int j = tid; j < n_dom; j += kBlkThreads) {
+      const u64 key = keys[first + j];
+      skeys[j] = key;
+      mx = key > mx ? key : mx;
+    }
+#pragma unroll 1
+    for (int off = 16; off >= 1; off >>= 1) {
+      const u64 o = __shfl_xor_sync(0xffffffffu, mx, off);
+      mx = o > mx ? o : mx;
+    }
+    if (lane == 0 && mx != 0) atomicMax(&sh_max, mx);
+  }
+  __syncthreads();
+  const u64 max_key = sh_max;
+
+  // ---- thresholds: T[c] = key of the k-th entry in "key descending" order, k_eq[c] = how many of its ties are taken
+  u64 pre[kSelMaxC];
+  unsigned int kq[kSelMaxC];
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) { pre[c] = 0; kq[c] = c < nC ? (unsigned)kk[c] : 0u; }
+#pragma unroll 1
+  for (int pass = kSelPasses - 1; pass >= 0; --pass) {
+    const int shift = pass * kDigitBits;
+    if ((max_key >> shift) == 0) {                       // this digit and those above are zero in every key
+      continue;
+    }
+    // candidates with the same prefix share a histogram; a key matches at most one prefix
+    int hsel[kSelMaxC];
+    uint32_t upre[kSelMaxC];
+    int n_hist = 0;
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) { hsel[c] = -1; upre[c] = 0xffffffffu; }
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC && kk[c] > 0) {
+      _Pragma("unroll") for (int d = 0; d < kSelMaxC; ++d)
+        if (d < c && hsel[c] < 0 && hsel[d] >= 0 && pre[d] == pre[c]) hsel[c] = hsel[d];
+      if (hsel[c] < 0) {
+        hsel[c] = n_hist;
+        _Pragma("unroll") for (int h = 0; h < kSelMaxC; ++h) if (h == n_hist) upre[h] = (uint32_t)pre[c];
+        ++n_hist;
+      }
+    }
+    for (int i = tid; i < n_hist * kBins; i += kBlkThreads) (&hist[0][0])[i] = 0;
+    __syncthreads();
+#pragma unroll 1
+    for (int base = lo; base < hi; base += 32) {
+      const bool in = base + lane < hi;
+      const u64 key = in ? skeys[base + lane] : 0ull;
+      const uint32_t up = (uint32_t)(key >> (shift + kDigitBits));
+      const uint32_t dig = (uint32_t)(key >> shift) & (kBins - 1);
+      unsigned int slot = 0xffffffffu;
+      _Pragma("unroll") for (int h = 0; h < kSelMaxC; ++h) if (up == upre[h]) slot = (unsigned)h * kBins + dig;
+      if (!in) slot = 0xffffffffu;
+      // small masses share their upper digits: the lanes that agree with lane 0 add once for all of them
+      const unsigned int slot0 = __shfl_sync(0xffffffffu, slot, 0);
+      const unsigned int same = __ballot_sync(0xffffffffu, slot == slot0);
+      if (slot == slot0) {
+        if (lane == 0 && slot != 0xffffffffu) atomicAdd(&(&hist[0][0])[slot], (unsigned)__popc(same));
+      } else if (slot != 0xffffffffu) {
+        atomicAdd(&(&hist[0][0])[slot], 1u);
+      }
+    }
+    __syncthreads();
+    // thread t owns the two bins kBins - 1 - 2 t and kBins - 2 - 2 t: counts from the top
+    unsigned int b_hi[kSelMaxC], sum2[kSelMaxC], incl[kSelMaxC];
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) {
+      b_hi[c] = sum2[c] = incl[c] = 0;
+      if (hsel[c] < 0) continue;
+      const uint2 two = *reinterpret_cast<const uint2*>(&hist[hsel[c]][kBins - 2 - 2 * tid]);
+      b_hi[c] = two.y;
+      sum2[c] = two.x + two.y;
+      unsigned int in = sum2[c];
+#pragma unroll 1
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, in, off);
+        if (lane >= off) in += t;
+      }
+      incl[c] = in;
+      if (lane == 31) wtot[c][warp] = in;
+    }
+    __syncthreads();
+    if (warp < kSelMaxC) {                               // exclusive prefix of the warps' totals, candidate = warp
+      const unsigned int v = wtot[warp][lane];
+      unsigned int in = v;
+#pragma unroll 1
+      for (int off = 1; off < 32; off <<= 1) {
+        const unsigned int t = __shfl_up_sync(0xffffffffu, in, off);
+        if (lane >= off) in += t;
+      }
+      wtot[warp][lane] = in - v;
+    }
+    __syncthreads();
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) {
+      if (hsel[c] < 0) continue;
+      const unsigned int above = wtot[c][warp] + incl[c] - sum2[c];
+      if (above < kq[c] && kq[c] <= above + sum2[c]) {   // exactly one thread: the k-th entry is in its bins
+        const bool upper = kq[c] <= above + b_hi[c];
+        sh_prefix[c] = (pre[c] << kDigitBits) | (u64)(upper ? kBins - 1 - 2 * tid : kBins - 2 - 2 * tid);
+        sh_k[c] = kq[c] - above - (upper ? 0u : b_hi[c]);
+      }
+    }
+    __syncthreads();
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (hsel[c] >= 0) { pre[c] = sh_prefix[c]; kq[c] = sh_k[c]; }
+  }
+  u64 T[kSelMaxC];
+  unsigned int k_eq[kSelMaxC];
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) {
+    T[c] = (c < nC && kk[c] > 0) ? pre[c] : ~0ull;       // k = 0: nothing is above or equal
+    k_eq[c] = (c < nC && kk[c] > 0) ? kq[c] : 0u;
+  }
+
+  // ---- ordered compaction
+  unsigned int gt[kSelMaxC] = {}, eq[kSelMaxC] = {};
+#pragma unroll 1
+  for (int j = lo + lane; j < hi; j += 32) {
+    const u64 key = skeys[j];
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) {
+      gt[c] += (key > T[c]) ? 1u : 0u;
+      eq[c] += (key == T[c]) ? 1u : 0u;
+    }
+  }
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC) {
+    const unsigned int g2 = __reduce_add_sync(0xffffffffu, gt[c]), e2 = __reduce_add_sync(0xffffffffu, eq[c]);
+    if (lane == 0) { w_gt[c][warp] = g2; w_eq[c][warp] = e2; }
+  }
+  __syncthreads();
+  if (warp < 2 * nC) {                                   // exclusive prefixes over the warps
+    unsigned int* row = (warp & 1) ? w_eq[warp >> 1] : w_gt[warp >> 1];
+    const unsigned int v = row[lane];
+    unsigned int in = v;
+#pragma unroll 1
+    for (int off = 1; off < 32; off <<= 1) {
+      const unsigned int t = __shfl_up_sync(0xffffffffu, in, off);
+      if (lane >= off) in += t;
+    }
+    row[lane] = in - v;
+  }
+  __syncthreads();
+  unsigned int pos[kSelMaxC], eq_run[kSelMaxC];
+  _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC) {
+    eq_run[c] = w_eq[c][warp];
+    pos[c] = w_gt[c][warp] + min(k_eq[c], eq_run[c]) + (list == 1 ? 1u : 0u);
+  }
+  const unsigned int lt_mask = (1u << lane) - 1u;
+#pragma unroll 1
+  for (int base = lo; base < hi; base += 32) {
+    const int j = base + lane;
+    const bool in = j < hi;
+    const u64 key = in ? skeys[j] : 0ull;
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC) {
+      bool take = in && key > T[c];
+      const bool is_eq = in && key == T[c];
+      const unsigned int beq = __ballot_sync(0xffffffffu, is_eq);
+      if (beq != 0u) {                                   // ties with the threshold are rare: taken in index order
+        take = take || (is_eq && eq_run[c] + __popc(beq & lt_mask) < k_eq[c]);
+        eq_run[c] += __popc(beq);
+      }
+      const unsigned int bt = __ballot_sync(0xffffffffu, take);
+      if (take) {
+        const unsigned int p = pos[c] + __popc(bt & lt_mask);
+        int32_t* out = (list == 0) ? (P.out.vs_cols + (size_t)slot_id[c] * P.out.kv_cap)
+                                   : (P.out.vs_offs + (size_t)slot_id[c] * P.out.ks_cap);
+        if ((int)p < cap) out[p] = first + j;
+      }
+      pos[c] += __popc(bt);
+    }
+  }
+  if (tid == 0) {
+    _Pragma("unroll") for (int c = 0; c < kSelMaxC; ++c) if (c < nC) {
+      if (list == 1) {
+        P.out.vs_offs[(size_t)slot_id[c] * P.out.ks_cap] = 0;
+        P.out.vs_count[4 * slot_id[c] + 1] = kk[c] + 1;
+      } else {
+        P.out.vs_count[4 * slot_id[c] + 0] = kk[c];
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------ pair counts (closed forms)
 __device__ __forceinline__ u64 pairs_dense(long long q0, long long q1) { return (u64)((q1 * (q1 + 1) - q0 * (q0 + 1)) / 2); }
 
@@ -409,9 +636,10 @@ __device__ __forceinline__ u64 pairs_a_shape(long long q0, long long q1, long lo
 }
 
 __device__ __forceinline__ u64 pairs_block_sparse(int qb_lo, int qb_hi, int k_b) {
-  u64 total = 0;
-  for (int qb = qb_lo; qb < qb_hi; ++qb) total += (u64)(min(k_b, qb + 1) - 1) * 4096ull + 2080ull;
-  return total;
+  // sum over query blocks of min(k_b, qb + 1) - 1 whole blocks and the diagonal one: the min is qb + 1 below m
+  const long long lo = qb_lo, hi = qb_hi, m = min(hi, max(lo, (long long)k_b));
+  const long long whole = (m * (m - 1) - lo * (lo - 1)) / 2 + (hi - m) * (long long)(k_b - 1);
+  return (u64)whole * 4096ull + (u64)(hi - lo) * 2080ull;
 }
 
 // ------------------------------------------------------------------------------------------ vertical-slash: D, coverage, pairs
@@ -437,15 +665,16 @@ __device__ __forceinline__ void vs_finish_block(const IdxParams& P, int job) {
   if (tid < RS_PROBE_GROUPS) cov[tid] = 0;
   if (tid == 0) extra_pairs = 0;
   __syncthreads();
-  for (int base = 0; base < n_offs; base += 8 * (int)blockDim.x) {     // eight independent loads in flight per thread
-    int ob[8];
+#pragma unroll 1
+  for (int base = 0; base < n_offs; base += 4 * (int)blockDim.x) {     // four independent loads in flight per thread
+    int ob[4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       const int i = base + u * (int)blockDim.x + tid;
       ob[u] = (i < n_offs) ? offs[i] : -1;
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < 4; ++u) {
       // offsets are ascending, so the lanes of a warp see runs of equal block diagonals: only the first lane of a run
       // touches the bitmap (32 lanes hammering one shared-memory word would serialise)
       const int d0 = ob[u] < 0 ? -1 : ob[u] >> 6, d1 = ob[u] < 0 ? -1 : (ob[u] + 63) >> 6;
@@ -456,10 +685,19 @@ __device__ __forceinline__ void vs_finish_block(const IdxParams& P, int job) {
     }
   }
   __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    for (int w = 0; w < 128; ++w) { wpre[w] = acc; acc += __popc(dbits[w]); }
-    wpre[128] = acc;
+  if (tid < 32) {                                        // four words per lane
+    int c4[4], sum = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { c4[u] = sum; sum += __popc(dbits[4 * tid + u]); }
+    int incl = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, off);
+      if (tid >= off) incl += t;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) wpre[4 * tid + u] = incl - sum + c4[u];
+    if (tid == 31) wpre[128] = incl;
   }
   __syncthreads();
   const int n_diag = wpre[128];
@@ -480,6 +718,7 @@ __device__ __forceinline__ void vs_finish_block(const IdxParams& P, int job) {
   const float* vert = P.vert + (size_t)item * RS_PROBE_GROUPS * P.n;
   const u64* vblk = P.vblk + (size_t)item * RS_PROBE_GROUPS * P.nb;
   u64 part[RS_PROBE_GROUPS] = {0, 0, 0, 0};
+#pragma unroll 1
   for (int kb = tid; kb < nbs; kb += blockDim.x) {
     const int d = qb_star - kb;
     if ((dbits[d >> 5] >> (d & 31)) & 1u) {
@@ -496,6 +735,7 @@ __device__ __forceinline__ void vs_finish_block(const IdxParams& P, int job) {
     const int w = x >> 5;
     return wpre[w] + __popc(dbits[w] & (0xffffffffu >> (31 - (x & 31))));
   };
+#pragma unroll 1
   for (int base = 0; base < n_cols; base += 4 * (int)blockDim.x) {      // four independent load chains per thread
     int jb[4];
 #pragma unroll
@@ -578,8 +818,17 @@ __device__ __forceinline__ void simple_stats_block(const IdxParams& P, int job) 
   const int n_off = window_covers_all ? q1 : win;
   const int n_col = window_covers_all ? 0 : min(n_sink, q1);
   u64 part[RS_PROBE_GROUPS] = {0, 0, 0, 0};
+  // four offsets per load where the masses are 16-byte aligned (rows are multiples of 64 entries)
+  const int n_vec = ((uintptr_t)slash & 15) == 0 ? n_off >> 2 : 0;
+#pragma unroll 2
+  for (int o = tid; o < n_vec; o += blockDim.x)
+#pragma unroll
+    for (int g = 0; g < RS_PROBE_GROUPS; ++g) {
+      const float4 m = reinterpret_cast<const float4*>(slash + (size_t)g * P.n)[o];
+      part[g] += (fx(m.x) + fx(m.y)) + (fx(m.z) + fx(m.w));
+    }
 #pragma unroll 4
-  for (int o = tid; o < n_off; o += blockDim.x)
+  for (int o = 4 * n_vec + tid; o < n_off; o += blockDim.x)
 #pragma unroll
     for (int g = 0; g < RS_PROBE_GROUPS; ++g) part[g] += fx(slash[(size_t)g * P.n + o]);
   for (int j = tid; j < n_col; j += blockDim.x)
@@ -607,16 +856,19 @@ template <int NT>
 __device__ int select_row(const float* score, int m, int take, int qb, int32_t* out, int cap, uint32_t* hist /*256*/,
                           uint32_t* sh /*8*/, unsigned int* wcnt /* 2 * NT / 32 */) {
   constexpr int NW = NT / 32;
+  constexpr int kU = NT > 256 ? 1 : 4;     // the evaluation runs it once per block: short code there, unrolled in the row kernel
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t T = 0xffffffffu, k_eq = 0;
   take = min(take, m);
   if (take > 0) {
     if (tid == 0) { sh[0] = 0; sh[1] = (uint32_t)take; }
+#pragma unroll 1
     for (int pass = 3; pass >= 0; --pass) {
       if (tid < 256) hist[tid] = 0;
       __syncthreads();
       const uint32_t prefix = sh[0];
       const int shift = pass * 8;
+#pragma unroll kU
       for (int i = tid; i < m; i += NT) {
         const uint32_t key = f32_order_key(score[i]);
         if (pass == 3 || (key >> (shift + 8)) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
@@ -655,6 +907,7 @@ __device__ int select_row(const float* score, int m, int take, int qb, int32_t* 
   const int chunk = (((m + NW - 1) / NW) + 31) / 32 * 32;
   const int lo = warp * chunk, hi = min(m, lo + chunk);
   unsigned int gt = 0, eq = 0;
+#pragma unroll kU
   for (int base = lo; base < hi; base += 32) {
     const int i = base + lane;
     const bool in = i < hi;
@@ -665,9 +918,11 @@ __device__ int select_row(const float* score, int m, int take, int qb, int32_t* 
   if (lane == 0) { wcnt[warp] = gt; wcnt[NW + warp] = eq; }
   __syncthreads();
   unsigned int gt_before = 0, eq_before = 0;
+#pragma unroll kU
   for (int w = 0; w < warp; ++w) { gt_before += wcnt[w]; eq_before += wcnt[NW + w]; }
   unsigned int pos = gt_before + min(k_eq, eq_before), eq_run = eq_before;
   const unsigned int lt_mask = (1u << lane) - 1u;
+#pragma unroll kU
   for (int base = lo; base < hi; base += 32) {
     const int i = base + lane;
     const bool in = i < hi && take > 0;
@@ -730,6 +985,7 @@ __device__ __forceinline__ void bs_eval_block(const IdxParams& P, int item, int 
   __shared__ u64 cov[RS_PROBE_GROUPS];
   if (P.stats == nullptr && P.choice != nullptr) return;    // materialise mode without stats: rows are built elsewhere
   int my_c = -1;
+#pragma unroll 1
   for (int c = 0, seen = 0; c < P.n_cand; ++c)
     if (P.lib[c].pattern == RS_BLOCK_SPARSE && seen++ == bs_index) my_c = c;
   if (my_c < 0 || (P.choice != nullptr && P.choice[item] != my_c)) return;
@@ -739,9 +995,11 @@ __device__ __forceinline__ void bs_eval_block(const IdxParams& P, int item, int 
   const int tid = threadIdx.x;
   if (P.bscore != nullptr) {
     const float* row = P.bscore + ((size_t)item * P.nb + qb) * P.nb;
+#pragma unroll 1
     for (int kb = tid; kb < qb; kb += NT) score[kb] = row[kb];
   } else {
     const float* row = P.bs_eval_ws + (size_t)item * P.nb;
+#pragma unroll 1
     for (int kb = tid; kb < qb; kb += NT) score[kb] = row[kb];
   }
   __syncthreads();
@@ -755,12 +1013,14 @@ __device__ __forceinline__ void bs_eval_block(const IdxParams& P, int item, int 
     const int cnt = select_row<NT>(score, qb, min(k_b, qb + 1) - 1, qb, sel, 1024, hist, sh, wcnt);
     if (P.choice == nullptr) {
       int32_t* dst = P.out.bs_blk + (size_t)slot * P.out.kb_cap;
+#pragma unroll 1
       for (int i = tid; i < cnt && i < P.out.kb_cap; i += NT) dst[i] = sel[i];
       if (tid == 0) P.out.bs_count[slot] = cnt;
     }
     if (P.stats != nullptr) {
       const u64* vblk = P.vblk + (size_t)item * RS_PROBE_GROUPS * P.nb;
       u64 part[RS_PROBE_GROUPS] = {0, 0, 0, 0};
+#pragma unroll 1
       for (int i = tid; i < cnt; i += NT)
 #pragma unroll
         for (int gg = 0; gg < RS_PROBE_GROUPS; ++gg) part[gg] += vblk[(size_t)gg * P.nb + sel[i]];
@@ -1239,7 +1499,8 @@ static int build_indices_impl(const rs_problem* p, const rs_candidate* lib, int 
   for (int c = 0; c < n_cand; ++c) { n_vs += (lib[c].pattern == RS_VERTICAL_SLASH); n_bs += (lib[c].pattern == RS_BLOCK_SPARSE); }
   const int sel_groups = choice ? 1 : (n_vs + kSelMaxC - 1) / kSelMaxC;
   const size_t sel_smem = (size_t)(choice ? 1 : kSelMaxC) * kBins * sizeof(unsigned int);
-  static rs_smem_attr sel_attr;
+  static rs_smem_attr sel_attr, sel_block_attr;
+  if (rs_ensure_dynamic_smem(sel_block_attr, rs_vs_select_block_kernel, kBlockSelMax * (int)sizeof(u64)) != RS_OK) return RS_ERR_CUDA;
   if (rs_ensure_dynamic_smem(sel_attr, rs_vs_select_kernel, (int)(kSelMaxC * kBins * sizeof(unsigned int))) != RS_OK)
     return RS_ERR_CUDA;
   const bool two_chains = any_vs && !skip_vs && (any_bs || stats != nullptr);
@@ -1250,7 +1511,10 @@ static int build_indices_impl(const rs_problem* p, const rs_candidate* lib, int 
     rc = rs_side_fork(stream, &side);
     if (rc != RS_OK) return rc;
   }
-  if (any_vs && !skip_vs) rs_vs_select_kernel<<<dim3(kSelCluster, 2 * n_items, sel_groups), kSelThreads, sel_smem, stream>>>(P);
+  if (any_vs && !skip_vs) {
+    if (P.n <= kBlockSelMax) rs_vs_select_block_kernel<<<dim3(2 * n_items, sel_groups), kBlkThreads, (size_t)P.n * sizeof(u64), stream>>>(P);
+    else rs_vs_select_kernel<<<dim3(kSelCluster, 2 * n_items, sel_groups), kSelThreads, sel_smem, stream>>>(P);
+  }
   const bool eval = any_bs && (choice == nullptr || stats != nullptr);
   {
     const int n_simple = stats != nullptr ? n_jobs : 0;
