@@ -108,6 +108,13 @@ int rs_side_join(cudaStream_t main) {
   return ok ? RS_OK : RS_ERR_CUDA;
 }
 
+void rs_side_release() {
+  if (t_side_dev < 0) return;
+  SideStream& S = g_side[t_side_dev];
+  t_side_dev = -1;
+  S.mu.unlock();
+}
+
 typedef CUresult (*encode_fn_t)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

@@ -231,20 +231,6 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
   const int tid = threadIdx.x, warp = warp_uniform(tid >> 5), lane = tid & 31;
 
-  // ---- work item
-  const int2 w = P.order[blockIdx.x];
-  const int item = w.x, tile = w.y;
-  const int s = item / P.Hq, h = item - s * P.Hq, g = h / P.group;
-  const int q0 = P.seg_bounds[s], q1 = P.seg_bounds[s + 1];
-  const int i0 = q0 + tile * kTileM;
-  const int rows_valid = min(kTileM, q1 - i0);
-  const int qb0 = i0 >> 6;
-  const bool has_hi = rows_valid > kChunk;
-  const int qb_last = has_hi ? qb0 + 1 : qb0;
-  const rs_candidate cand = (P.choice != nullptr) ? P.lib[P.choice[item]] : rs_candidate{RS_DENSE, 0, 0, 0};
-  const int pattern = cand.pattern;
-  const int nb_words = (qb_last >> 5) + 1;
-
   // ---- shared memory carve-up
   const int list_cap = (P.n >> 6) + 64;
   uint16_t* list = reinterpret_cast<uint16_t*>(sm + SmemLayout::end_tiles);
@@ -283,6 +269,22 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = (uint32_t)warp_uniform(misc[0]);
+
+  // ---- work item: the first thing that earlier kernels have written
+  rs_grid_wait();
+  rs_grid_trigger();
+  const int2 w = P.order[blockIdx.x];
+  const int item = w.x, tile = w.y;
+  const int s = item / P.Hq, h = item - s * P.Hq, g = h / P.group;
+  const int q0 = P.seg_bounds[s], q1 = P.seg_bounds[s + 1];
+  const int i0 = q0 + tile * kTileM;
+  const int rows_valid = min(kTileM, q1 - i0);
+  const int qb0 = i0 >> 6;
+  const bool has_hi = rows_valid > kChunk;
+  const int qb_last = has_hi ? qb0 + 1 : qb0;
+  const rs_candidate cand = (P.choice != nullptr) ? P.lib[P.choice[item]] : rs_candidate{RS_DENSE, 0, 0, 0};
+  const int pattern = cand.pattern;
+  const int nb_words = (qb_last >> 5) + 1;
 
   // Q tile load goes out before the chunk list is built.
   if (tid == 0) {
@@ -717,6 +719,8 @@ rs_attn_prepare_kernel(AttnParams P, int n_groups, int per_group, int n_bins, in
                        int pack_blocks, const __nv_bfloat16* K, const __nv_bfloat16* V, __nv_bfloat16* Kp,
                        __nv_bfloat16* Vp) {
   extern __shared__ int hist[];
+  rs_grid_wait();
+  rs_grid_trigger();
   if ((int)blockIdx.x >= n_groups) {
     const int pb = blockIdx.x - n_groups;
     const int item = pb / pack_blocks;
@@ -853,11 +857,11 @@ int enqueue_attn(const rs_problem* p, const void* Q, const void* K, const void* 
   const int pack_blocks = pack ? (P.kv_pad + 63) / 64 : 0;
   const size_t kv_bytes = 2ull * (size_t)P.Hkv * (size_t)P.n * RS_HEAD_DIM * sizeof(__nv_bfloat16);
   const int n_groups = (kv_bytes <= kL2ResidentBytes || n_work % P.Hkv != 0) ? 1 : P.Hkv;
-  rs_attn_prepare_kernel<<<n_groups + pack_blocks * sc.n_items, 1024, (n_bins + 1) * sizeof(int), stream>>>(
+  rs_launch_dependent(rs_attn_prepare_kernel, n_groups + pack_blocks * sc.n_items, 1024, (n_bins + 1) * sizeof(int), stream,
       P, n_groups, n_work / n_groups, n_bins, sc.cost, sc.items, sc.order, pack_blocks,
       reinterpret_cast<const __nv_bfloat16*>(K), reinterpret_cast<const __nv_bfloat16*>(V), sc.Kp, sc.Vp);
   if (rs_ensure_dynamic_smem(g_attn_smem, rs_attn_kernel, 116 * 1024) != RS_OK) return RS_ERR_CUDA;
-  rs_attn_kernel<<<n_work, kThreads, attn_smem_bytes(P.n), stream>>>(tmQ, tmK, tmV, tmKp, tmVp, P);
+  rs_launch_dependent(rs_attn_kernel, n_work, kThreads, attn_smem_bytes(P.n), stream, tmQ, tmK, tmV, tmKp, tmVp, P);
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
 

@@ -11,6 +11,7 @@ rs_certificate_kernel(int n_keys, int group, const float* lse_sel, const float* 
   __shared__ double s_sum[8];
   __shared__ float s_max[8];
   __shared__ int s_ok;
+  rs_grid_wait();
   if (threadIdx.x == 0) s_ok = 0;
   __syncthreads();
   const int h = blockIdx.x;
@@ -66,7 +67,7 @@ extern "C" int rs_certificate(int n_q_heads, int n_kv_heads, int n_keys, const f
                               float* cert_head, int32_t* status, void* stream_) {
   if (n_q_heads <= 0 || n_kv_heads <= 0 || n_q_heads % n_kv_heads != 0 || n_keys <= 0 || n_rows <= 0 || !lse_sel || !lse_full || !rows || !vmax_head)
     return RS_ERR_INVALID_ARG;
-  rs_certificate_kernel<<<n_q_heads, 256, 0, (cudaStream_t)stream_>>>(n_keys, n_q_heads / n_kv_heads, lse_sel, lse_full, rows, n_rows, vmax_head,
+  rs_launch_dependent(rs_certificate_kernel, n_q_heads, 256, 0, (cudaStream_t)stream_, n_keys, n_q_heads / n_kv_heads, lse_sel, lse_full, rows, n_rows, vmax_head,
                                                                      onorm, delta_q, m_row, cert_row, cert_tight, m_head,
                                                                      cert_head, status);
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;

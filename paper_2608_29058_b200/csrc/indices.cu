@@ -97,6 +97,8 @@ __global__ void rs_vblk_kernel(IdxParams P) {
 __global__ void __launch_bounds__(256)
 rs_vs_keys_kernel(IdxParams P, int fuse_vblk) {
   __shared__ u64 half_sum[8][RS_PROBE_GROUPS];
+  rs_grid_wait();
+  rs_grid_trigger();
   const int item = blockIdx.y >> 1, list = blockIdx.y & 1;
   const int s = item / P.Hq;
   const int q1 = P.seg_bounds[s + 1];
@@ -412,6 +414,8 @@ rs_vs_select_block_kernel(IdxParams P) {
   __shared__ unsigned int wtot[kSelMaxC][kBlkWarps], w_gt[kSelMaxC][kBlkWarps], w_eq[kSelMaxC][kBlkWarps];
   __shared__ u64 sh_prefix[kSelMaxC], sh_max;
   __shared__ unsigned int sh_k[kSelMaxC];
+  rs_grid_wait();
+  rs_grid_trigger();
   const int list = blockIdx.x & 1, item = blockIdx.x >> 1;
   int cand_id[kSelMaxC] = {}, slot_id[kSelMaxC] = {}, kk[kSelMaxC] = {};
   int nC = 0;
@@ -1042,6 +1046,8 @@ __device__ __forceinline__ void bs_eval_block(const IdxParams& P, int item, int 
 __global__ void __launch_bounds__(kFinishThreads)
 rs_finish_eval_kernel(IdxParams P, int n_finish, int n_items) {
   extern __shared__ float score[];      // [nb], used by the block-sparse part
+  rs_grid_wait();
+  rs_grid_trigger();
   if ((int)blockIdx.x < n_finish) {
     vs_finish_block(P, blockIdx.x);
   } else {
@@ -1157,6 +1163,8 @@ __device__ __forceinline__ void bs_row_warp(const IdxParams& P, int qb, int h) {
 __global__ void __launch_bounds__(256)
 rs_bs_rows_kernel(IdxParams P, int n_short) {
   extern __shared__ float score[];      // [nb], used by the block-per-row part
+  rs_grid_wait();
+  rs_grid_trigger();
   const int n_warp_blocks = (n_short + 7) / 8;
   const int h = blockIdx.y;
   if ((int)blockIdx.x < n_warp_blocks) {
@@ -1173,6 +1181,8 @@ __global__ void __launch_bounds__(256)
 rs_bs_scores_kernel(IdxParams P) {
   __shared__ float As[64][33], Bs[64][33];
   __shared__ int any_bs;
+  rs_grid_wait();
+  rs_grid_trigger();
   const int kt = blockIdx.x, qt = blockIdx.y, h = blockIdx.z;
   if (kt > qt) return;
   const int tid = threadIdx.x;
@@ -1506,13 +1516,13 @@ static int build_indices_impl(const rs_problem* p, const rs_candidate* lib, int 
   const bool two_chains = any_vs && !skip_vs && (any_bs || stats != nullptr);
   cudaStream_t side = stream;
   // the ranking keys (and with them the block sums both chains read) come before the fork
-  if (any_vs && !skip_vs) rs_vs_keys_kernel<<<dim3((P.n + 255) / 256, 2 * n_items), 256, 0, stream>>>(P, fuse_vblk ? 1 : 0);
+  if (any_vs && !skip_vs) rs_launch_dependent(rs_vs_keys_kernel, dim3((P.n + 255) / 256, 2 * n_items), 256, 0, stream, P, fuse_vblk ? 1 : 0);
   if (two_chains) {
     rc = rs_side_fork(stream, &side);
     if (rc != RS_OK) return rc;
   }
   if (any_vs && !skip_vs) {
-    if (P.n <= kBlockSelMax) rs_vs_select_block_kernel<<<dim3(2 * n_items, sel_groups), kBlkThreads, (size_t)P.n * sizeof(u64), stream>>>(P);
+    if (P.n <= kBlockSelMax) rs_launch_dependent(rs_vs_select_block_kernel, dim3(2 * n_items, sel_groups), kBlkThreads, (size_t)P.n * sizeof(u64), stream, P);
     else rs_vs_select_kernel<<<dim3(kSelCluster, 2 * n_items, sel_groups), kSelThreads, sel_smem, stream>>>(P);
   }
   const bool eval = any_bs && (choice == nullptr || stats != nullptr);
@@ -1525,11 +1535,11 @@ static int build_indices_impl(const rs_problem* p, const rs_candidate* lib, int 
   if (any_bs && choice != nullptr) {
     if (bscore == nullptr) {
       const int nt = (nb + 63) / 64;
-      rs_bs_scores_kernel<<<dim3(nt, nt, P.Hq), 256, 0, side>>>(P);
+      rs_launch_dependent(rs_bs_scores_kernel, dim3(nt, nt, P.Hq), 256, 0, side, P);
     }
     // short rows one warp each; rows with more than 1024 candidate blocks one thread block each
     const int n_short = nb < kWarpRowMax + 1 ? nb : kWarpRowMax + 1;       // query blocks 0 .. 1024
-    rs_bs_rows_kernel<<<dim3((n_short + 7) / 8 + (nb - n_short), P.Hq), 256, (size_t)nb * sizeof(float), side>>>(P, n_short);
+    rs_launch_dependent(rs_bs_rows_kernel, dim3((n_short + 7) / 8 + (nb - n_short), P.Hq), 256, (size_t)nb * sizeof(float), side, P, n_short);
   }
   if (two_chains) {
     rc = rs_side_join(stream);
@@ -1540,7 +1550,7 @@ static int build_indices_impl(const rs_problem* p, const rs_candidate* lib, int 
     const int n_finish = any_vs && !skip_vs ? n_jobs : 0;
     const int n_eval = eval ? n_items * n_bs : 0;
     if (n_finish + n_eval > 0)
-      rs_finish_eval_kernel<<<n_finish + n_eval, kFinishThreads, (size_t)nb * sizeof(float), stream>>>(P, n_finish, n_items);
+      rs_launch_dependent(rs_finish_eval_kernel, n_finish + n_eval, kFinishThreads, (size_t)nb * sizeof(float), stream, P, n_finish, n_items);
   }
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }

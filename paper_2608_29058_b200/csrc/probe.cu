@@ -119,6 +119,8 @@ rs_probe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 #pragma unroll
   for (int i = 0; i < 2; ++i) { bar_tfull[i] = smem_u32(&bars[1 + 2 * kStages + i]); bar_tempty[i] = smem_u32(&bars[3 + 2 * kStages + i]); }
 
+  rs_grid_wait();
+  rs_grid_trigger();
   if (tid == 0) {
     mbar_init(bar_q, 1);
     for (int i = 0; i < kStages; ++i) { mbar_init(bar_full[i], 1); mbar_init(bar_empty[i], do_pool ? 3 : 1); }
@@ -678,6 +680,8 @@ __global__ void __launch_bounds__(256)
 rs_pool_q_routed_kernel(ProbeParams P, const __nv_bfloat16* __restrict__ Q, float* __restrict__ out, rs_candidate_list L,
                         const int32_t* __restrict__ choice) {
   __shared__ float red[16][128 + 4];
+  rs_grid_wait();
+  rs_grid_trigger();
   const int nb = P.n >> 6;
   const int h = blockIdx.y;
   int s = -1;
@@ -714,7 +718,7 @@ extern "C" int rs_pool_queries(const rs_problem* p, const void* Q, const rs_cand
   for (int c = 0; c < n_cand; ++c) { L.pattern[c] = lib[c].pattern; any_bs |= lib[c].pattern == RS_BLOCK_SPARSE; }
   if (!any_bs) return RS_OK;                            // no block-sparse candidate: nothing can be routed to it
   const int nb = P.n >> 6;
-  rs_pool_q_routed_kernel<<<dim3((nb + kPoolRun - 1) / kPoolRun, P.Hq), 256, 0, (cudaStream_t)stream_>>>(
+  rs_launch_dependent(rs_pool_q_routed_kernel, dim3((nb + kPoolRun - 1) / kPoolRun, P.Hq), 256, 0, (cudaStream_t)stream_,
       P, reinterpret_cast<const __nv_bfloat16*>(Q), qpool, L, choice);
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
@@ -790,7 +794,7 @@ static int probe_impl(const rs_problem* p, const void* Q, const void* K, const v
     if (rc != RS_OK) return rc;
   }
   dim3 grid(w.n_splits, w.n_units);
-  rs_probe_kernel<1><<<grid, kThreads1, SmemT<1>::total, stream>>>(tmQ, tmK, P);
+  rs_launch_dependent(rs_probe_kernel<1>, grid, kThreads1, SmemT<1>::total, stream, tmQ, tmK, P);
   if (vmax) {
     float* blockmax = reinterpret_cast<float*>(wsb + w.blockmax);
     rs_vnorm_block_kernel<<<(unsigned)(P.Hkv * nb), 256, 0, side>>>(reinterpret_cast<const __nv_bfloat16*>(V), blockmax, P.Hkv * nb);
@@ -800,10 +804,12 @@ static int probe_impl(const rs_problem* p, const void* Q, const void* K, const v
   }
   if (pool_all)
     rs_pool_kernel<<<(unsigned)(P.Hq * nb), 256, 0, side>>>(reinterpret_cast<const __nv_bfloat16*>(Q), qpool, P.Hq * nb);
-  rs_probe_kernel<2><<<grid, kThreads2, SmemT<2>::total, stream>>>(tmQ, tmK32, P);
-  if (use_side) {
+  rs_launch_dependent(rs_probe_kernel<2>, grid, kThreads2, SmemT<2>::total, stream, tmQ, tmK32, P);
+  if (pool_all) {
     rc = rs_side_join(stream);
     if (rc != RS_OK) return rc;
+  } else if (use_side) {
+    rs_side_release();                       // the wait in front of pass 2 has covered all of the side stream's work
   }
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }

@@ -125,6 +125,8 @@ rs_route_kernel(const __grid_constant__ RouteArgs A) {
   __shared__ long long sh_total;
   __shared__ int sh_feasible, sh_fallback;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  rs_grid_wait();
+  rs_grid_trigger();
   const int n_pairs = A.n_items * A.n_cand;
   const bool cached = n_cache > 0;
   if (cached) {
@@ -624,6 +626,6 @@ extern "C" int rs_route(const rs_problem* p, const rs_candidate* lib, int n_cand
                       (n_pairs <= kSortPairs ? (size_t)kSortPairs * (sizeof(double) + 4) + (size_t)n_pairs * (sizeof(double) + 1) : 0);
   static rs_smem_attr route_attr;
   if (rs_ensure_dynamic_smem(route_attr, rs_route_kernel, 225 * 1024) != RS_OK) return RS_ERR_CUDA;
-  rs_route_kernel<<<1, kThreads, smem, (cudaStream_t)stream_>>>(A);
+  rs_launch_dependent(rs_route_kernel, 1, kThreads, smem, (cudaStream_t)stream_, A);
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }

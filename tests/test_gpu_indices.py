@@ -155,3 +155,31 @@ def test_argument_checks():
     z = np.zeros((1, 2, 4, 256), np.float32)
     with pytest.raises(rs.RouteSparseError):
         gpu_build(p, lib_c, z, z, None, None, None, None)
+
+
+@pytest.mark.parametrize("kind", ["spread", "ties", "zeros", "large"])
+@pytest.mark.parametrize("n", [64, 1088, 16384, 16448])
+def test_line_selection_at_the_edges_of_its_two_kernels(n, kind):
+    """Columns and offsets are the k largest integer keys, ties to the lower index: lists of one block and of a cluster of
+    blocks (up to 16384 keys and above), five budgets (two groups of candidates) from nothing to every line, masses spread
+    over the digits, full of ties, all zero, and with the upper digits in use."""
+    rng = np.random.default_rng(n + len(kind))
+    mass = lambda: {"spread": 2.0 ** rng.uniform(-34, 3, (1, 1, 4, n)), "ties": rng.integers(0, 5, (1, 1, 4, n)) / 64.0,
+                    "zeros": np.zeros((1, 1, 4, n)), "large": rng.choice([0.0, 2.0 ** -20, 3.0, 700.0], (1, 1, 4, n))}[kind].astype(np.float32)
+    vert, slash = mass(), mass()
+    budgets = [(0, 1), (1, 2), (37, 100), (n // 2 + 1, n - 1), (n, n)]
+    lib = [C(PT.VERTICAL_SLASH, kv, ks) for kv, ks in budgets] + [C(PT.DENSE)]
+    p = rs.Problem(1, 1, n)
+    idx, _ = gpu_build(p, c_library(lib), vert, slash, None, None, None, None)
+    key = lambda m: np.floor(m[0, 0].astype(np.float64) * 2.0 ** 32).astype(np.uint64).sum(axis=0)
+    order = lambda k: np.lexsort((np.arange(len(k)), -k.astype(np.int64)))
+    cols, offs = order(key(vert)), 1 + order(key(slash)[1:])
+    cnt = idx.vs_count.cpu().numpy()
+    for c, (kv, ks) in enumerate(budgets):
+        V, S = np.sort(cols[:kv]), np.concatenate([[0], np.sort(offs[:ks - 1])])
+        D = np.unique(np.concatenate([S // 64, (S + 63) // 64]))
+        D = D[D < n // 64]
+        assert cnt[c, :3].tolist() == [len(V), len(S), len(D)], (c, cnt[c], len(V), len(S), len(D))
+        assert np.array_equal(idx.vs_cols[c, :len(V)].cpu().numpy(), V)
+        assert np.array_equal(idx.vs_offs[c, :len(S)].cpu().numpy(), S)
+        assert np.array_equal(idx.vs_diag[c, :len(D)].cpu().numpy(), D)

@@ -323,3 +323,34 @@ def test_two_layers_on_two_streams():
         rs.check_status(layers[k].status, f"stream {k}")
         assert torch.equal(layers[k].O, want[k][0]) and torch.equal(layers[k].choice, want[k][1])
         assert torch.equal(layers[k].lse_sel, want[k][2])
+
+
+@pytest.mark.parametrize("n,Hq,Hkv,bounds", [(64, 1, 1, [0, 64]), (1280, 8, 2, [0, 512, 1280]), (4096, 2, 1, [0, 4096])])
+def test_passes_back_to_back_equal_passes_on_their_own(n, Hq, Hkv, bounds):
+    """The kernels of a pass start while the one in front of them drains.  Passes over three inputs, enqueued without a
+    synchronisation between them, leave what each pass leaves when the GPU is idle around it, bit for bit."""
+    p = rs.Problem(Hq, Hkv, n, bounds)
+    lib = [(rs.RS_A_SHAPE, 8, 4 * n if n < 256 else 128), (rs.RS_VERTICAL_SLASH, 32, 48), (rs.RS_BLOCK_SPARSE, 3, 0), (rs.RS_DENSE, 0, 0)]
+    layer = rs.RoutedPrefillLayer(p, lib, rs.RouteConfig(budget_frac=0.4, cert_max=0.5))
+    inputs = []
+    for seed in (301, 302, 303):
+        L = make_layer(tiny_spec(seed, n, Hq, Hkv))
+        inputs.append([dev_bf16(L[x]) for x in "QKV"])
+    read = lambda: [t.clone() for t in (layer.O, layer.lse_sel, layer.onorm, layer.choice, layer.m_row, layer.cert_head, layer.stats)]
+    alone = []
+    for x in inputs:
+        torch.cuda.synchronize()
+        layer.forward(*x)
+        torch.cuda.synchronize()
+        alone.append(read())
+    for _ in range(10):
+        together = []
+        for x in inputs:
+            layer.forward(*x)
+            together.append(read())
+        for a, b in zip(alone, together):
+            assert all(torch.equal(u, v) for u, v in zip(a, b))
+        for x in inputs[:2]:                       # nothing of this stream's between the passes
+            layer.forward(*x)
+        assert all(torch.equal(u, v) for u, v in zip(alone[1], read()))
+    rs.check_status(layer.status, "back to back")
