@@ -39,6 +39,7 @@ struct AttnParams {
   int kv_pad;                 // rows per slot of the packed vertical K/V
   int vs_eval_layout;         // 1: vertical-slash lists sit in the evaluation layout, slot = item * n_cand + candidate
   const int2* order;          // [n_work] (item, tile in segment), heavy first
+  int split;                  // CTAs that share a tile's chunks (a cluster; 1: none)
   void* O;
   int o_f32;
   float* lse;
@@ -220,6 +221,109 @@ __device__ __noinline__ float3 rs_raise_and_exp(uint32_t t_x, float sl2, float m
   return make_float3(m_run, l_run, sum);
 }
 
+// ------------------------------------------------------------------------------------------ tiles shared by a cluster
+// When a launch has too few tiles for the chip, `split` CTAs of a cluster take every split-th chunk of a tile and each ends
+// with its own (m, l, O).  Rank q owns rows [q 128 / split, ...): the rows' partial results travel to it through
+// distributed shared memory, into the K / V rings that nobody uses any more, and it forms
+// O = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k.  All threads of all ranks call it.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__device__ __noinline__ void combine_split(const AttnParams& P, uint8_t* sm, unsigned long long* stat_mem, int split, int rank,
+                                           int h, int i0, int rows_valid, float m_run, float l_run, bool has_o,
+                                           uint32_t tmem) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int per = kTileM / split;                       // rows of an owner
+  float* recv = reinterpret_cast<float*>(sm + SmemLayout::k);          // [split][per][128], 16-byte pieces swizzled by row
+  float2* stat = reinterpret_cast<float2*>(stat_mem);                  // [split][per]
+  __syncthreads();
+  cluster_sync();                                       // every rank's products are done, its rings are free
+  if (warp >= 2) {
+    const int quad = warp & 3, r = quad * 32 + lane, owner = r / per, lr = r - owner * per;
+    const uint32_t dst = map_to_rank(smem_u32(recv + ((size_t)rank * per + lr) * RS_HEAD_DIM), (uint32_t)owner);
+    const uint32_t dst_stat = map_to_rank(smem_u32(stat + rank * per + lr), (uint32_t)owner);
+    if (!has_o) { m_run = -INFINITY; l_run = 0.f; }
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(dst_stat), "f"(m_run), "f"(l_run) : "memory");
+    if (has_o) {
+      const uint32_t t_o = tmem + ((uint32_t)(quad * 32) << 16) + kColO;
+#pragma unroll 1
+      for (int c = 0; c < RS_HEAD_DIM; c += 32) {
+        uint32_t v[32];
+        tmem_ld32(t_o + (uint32_t)c, v);
+        tc_wait_ld32(v);
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+          asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                       ::"r"(dst + 16u * (uint32_t)(((c >> 2) + x) ^ (lr & 7))), "r"(v[4 * x]), "r"(v[4 * x + 1]),
+                         "r"(v[4 * x + 2]), "r"(v[4 * x + 3]) : "memory");
+      }
+    }
+  }
+  cluster_sync();                                       // all partial results have arrived
+  if (warp < 2) return;
+  // split threads per owned row, 128 / split columns each
+  const int t = tid - 64, lr = t / split, part = t - lr * split, r = rank * per + lr;
+  const int cols = RS_HEAD_DIM / split;
+  float M = -INFINITY;
+  for (int k = 0; k < split; ++k) M = fmaxf(M, stat[k * per + lr].x);
+  float L = 0.f, wk[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    wk[k] = 0.f;
+    if (k >= split) continue;
+    const float2 ml = stat[k * per + lr];
+    if (ml.x == -INFINITY) continue;                    // nothing of this row there
+    wk[k] = fast_exp2(ml.x - M);
+    L = fmaf(ml.y, wk[k], L);
+  }
+  const float inv = L > 0.f ? 1.0f / L : 0.f;
+  const bool valid = r < rows_valid;
+  const size_t row = (size_t)h * P.n + (size_t)(i0 + r);
+  float ss = 0.f;
+#pragma unroll 1
+  for (int c = part * cols; c < (part + 1) * cols; c += 8) {
+    float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k >= split || wk[k] == 0.f) continue;
+      const float* src = recv + ((size_t)k * per + lr) * RS_HEAD_DIM;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const float4 o = *reinterpret_cast<const float4*>(src + 4 * (((c >> 2) + x) ^ (lr & 7)));
+        f[4 * x] = fmaf(wk[k], o.x, f[4 * x]); f[4 * x + 1] = fmaf(wk[k], o.y, f[4 * x + 1]);
+        f[4 * x + 2] = fmaf(wk[k], o.z, f[4 * x + 2]); f[4 * x + 3] = fmaf(wk[k], o.w, f[4 * x + 3]);
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < 8; ++x) { f[x] *= inv; ss = fmaf(f[x], f[x], ss); }
+    if (!valid) continue;
+    if (P.o_f32) {
+      float4* d = reinterpret_cast<float4*>(reinterpret_cast<float*>(P.O) + row * RS_HEAD_DIM + c);
+      d[0] = make_float4(f[0], f[1], f[2], f[3]);
+      d[1] = make_float4(f[4], f[5], f[6], f[7]);
+    } else {
+      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(P.O) + row * RS_HEAD_DIM + c) =
+          make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+    }
+  }
+  for (int off = 1; off < split; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+  if (valid && part == 0) {
+    P.lse[row] = (M + log2f(L)) * 0.6931471805599453f;
+    if (P.onorm != nullptr) P.onorm[row] = sqrtf(ss);
+  }
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
 rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKp,
@@ -273,7 +377,9 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   // ---- work item: the first thing that earlier kernels have written
   rs_grid_wait();
   rs_grid_trigger();
-  const int2 w = P.order[blockIdx.x];
+  const int split = P.split;
+  const int rank = split > 1 ? (int)cluster_rank() : 0;      // takes chunks rank, rank + split, ...
+  const int2 w = P.order[split > 1 ? blockIdx.x / split : blockIdx.x];
   const int item = w.x, tile = w.y;
   const int s = item / P.Hq, h = item - s * P.Hq, g = h / P.group;
   const int q0 = P.seg_bounds[s], q1 = P.seg_bounds[s + 1];
@@ -430,7 +536,8 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   }
   __syncthreads();
   const int n_block = warp_uniform(misc[2]), n_vert = (warp_uniform(misc[3]) + kChunk - 1) / kChunk;     // misc[3]: visible gathered columns
-  const int n_chunks = n_block + n_vert;
+  const int n_chunks = (n_block + n_vert - rank + split - 1) / split;
+  float m_run = -INFINITY, l_run = 0.f;      // softmax threads: reference and sum of their row
   // =========================================================================================== roles
   // Everything below is pipelined per 64-key chunk; chunk c uses slot c & 1 of the K / V rings, of the two 64-column
   // score buffers in TMEM and of the barrier pairs, in phase (c >> 1) & 1.  While the softmax warps work on chunk c the
@@ -459,13 +566,13 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           const uint32_t slot = (uint32_t)(ch & 1), ph = (uint32_t)((ch >> 1) & 1);
           ok = mbar_wait(bar_ve + 8u * slot, ph ^ 1u, abort_flag); site = 2;
           if (!ok) break;
-          load_chunk(ch, base + SmemLayout::v + slot * 8192u, bar_vf + 8u * slot, &tmV, &tmVp);
+          load_chunk(rank + split * ch, base + SmemLayout::v + slot * 8192u, bar_vf + 8u * slot, &tmV, &tmVp);
         }
         if (i < n_chunks) {
           const uint32_t slot = (uint32_t)(i & 1), ph = (uint32_t)((i >> 1) & 1);
           ok = mbar_wait(bar_ke + 8u * slot, ph ^ 1u, abort_flag); site = 1;
           if (!ok) break;
-          load_chunk(i, base + SmemLayout::k + slot * 8192u, bar_kf + 8u * slot, &tmK, &tmKp);
+          load_chunk(rank + split * i, base + SmemLayout::k + slot * 8192u, bar_kf + 8u * slot, &tmK, &tmKp);
         }
       }
       if (!ok) { rs_report(P.status, RS_ERR_TIMEOUT, site); *abort_flag = 1; }
@@ -540,7 +647,6 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const uint32_t t_s = tmem + lane_addr + kColS, t_o = tmem + lane_addr + kColO;
     const float sl2 = P.scale_log2e;
     const float NEG_INF = -INFINITY;
-    float m_run = NEG_INF, l_run = 0.f;
     const int* vcols = P.idx.vs_cols + (size_t)vs_slot * P.idx.kv_cap;
     bool ok = true;
     uint32_t v[32], v2[32];
@@ -557,8 +663,9 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       {
         int mode = -1, j0 = 0, edge = 0, vbase = 0;
         unsigned long long vk = 0ull, vd = 0ull;
-        if (ch < n_block) {
-          const uint32_t e = list[ch];
+        const int gch = rank + split * ch;
+        if (gch < n_block) {
+          const uint32_t e = list[gch];
           if (!(e & (half ? F_HI : F_LO))) {
             mode = 0;
           } else if (e & (F_CAUSAL | F_EDGE)) {
@@ -567,7 +674,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             edge = (e & F_EDGE) ? 1 : 0;
           }
         } else {
-          const int vch = ch - n_block;
+          const int vch = gch - n_block;
           vbase = vch * kChunk;
           if (vch < kMaskChunks) {
             vk = vkeep[vch * 2 + half];
@@ -622,7 +729,9 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
 
     if (ok) ok = mbar_wait(bar_o, 0, abort_flag);
-    if (ok) {
+    if (ok && split > 1) {
+      tc_fence_after();                       // combined below
+    } else if (ok) {
       tc_fence_after();
       const float inv = (l_run > 0.f) ? 1.0f / l_run : 0.f;
       const bool valid = r < rows_valid;
@@ -660,11 +769,13 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
   }
 
+  if (split > 1) combine_split(P, sm, vkeep, split, rank, h, i0, rows_valid, m_run, l_run, n_chunks > 0, tmem);
+
   tc_fence_before();
   __syncthreads();
   if (tid == 0 && P.counters != nullptr) {
     atomicAdd(&P.counters[0], (unsigned long long)n_chunks);
-    atomicAdd(&P.counters[1], 1ull);
+    if (rank == 0) atomicAdd(&P.counters[1], 1ull);
   }
   if (warp == 1) {
     tc_fence_after();
@@ -809,6 +920,14 @@ constexpr size_t kL2ResidentBytes = 96ull << 20;     // K + V of all heads below
 // vertical-slash items, the packed K / V rows of the gathered columns.
 struct AttnScratch { int* cost; int2* items; int2* order; __nv_bfloat16 *Kp, *Vp; int kv_pad; int n_work, n_items; };
 
+// CTAs per tile: as many as two per SM allow, as long as each keeps eight chunks of the longest tile.  From 2048 keys on:
+// below, the fixed cost of a tile and of the combination is what a launch consists of.
+int attn_split(int n, int n_work) {
+  int split = 1;
+  while (split < 8 && n >= 2048 && 2 * split * n_work <= 2 * 148 && n / 64 >= 16 * split) split *= 2;
+  return split;
+}
+
 // Enqueues the preparation kernel (work list, gather of the vertical columns) and the attention launch.  Arguments are checked
 // by the callers; `sc` says where the scratch lives (caller workspace or the library's built-in array).
 int enqueue_attn(const rs_problem* p, const void* Q, const void* K, const void* V, const rs_candidate* lib, int n_cand,
@@ -861,7 +980,9 @@ int enqueue_attn(const rs_problem* p, const void* Q, const void* K, const void* 
       P, n_groups, n_work / n_groups, n_bins, sc.cost, sc.items, sc.order, pack_blocks,
       reinterpret_cast<const __nv_bfloat16*>(K), reinterpret_cast<const __nv_bfloat16*>(V), sc.Kp, sc.Vp);
   if (rs_ensure_dynamic_smem(g_attn_smem, rs_attn_kernel, 116 * 1024) != RS_OK) return RS_ERR_CUDA;
-  rs_launch_dependent(rs_attn_kernel, n_work, kThreads, attn_smem_bytes(P.n), stream, tmQ, tmK, tmV, tmKp, tmVp, P);
+  P.split = attn_split(P.n, n_work);
+  rs_launch_dependent_cluster(P.split, rs_attn_kernel, n_work * P.split, kThreads, attn_smem_bytes(P.n), stream, tmQ, tmK, tmV,
+                              tmKp, tmVp, P);
   return cudaGetLastError() == cudaSuccess ? RS_OK : RS_ERR_CUDA;
 }
 

@@ -273,14 +273,21 @@ static inline size_t rs_align_up(size_t x, size_t a) { return (x + a - 1) / a * 
 // where everything it reads comes from the kernel in front of it or from in front of that one's own wait (or is awaited
 // through an event).
 template <typename... P, typename... A>
-static inline void rs_launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+static inline void rs_launch_dependent_cluster(int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                               cudaStream_t stream, A&&... args) {
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cfg.attrs = &attr; cfg.numAttrs = 1;
+  cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);      // errors surface through cudaGetLastError
+}
+template <typename... P, typename... A>
+static inline void rs_launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+  rs_launch_dependent_cluster(1, kernel, grid, block, smem, stream, static_cast<A&&>(args)...);
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) is a per-device setting: it is applied once per (kernel, device)

@@ -211,3 +211,37 @@ def test_dense_when_scores_climb(steps, offset):
     assert_attention_close(O[0].cpu().numpy(), Oo, f"steps {steps} offset {offset}")
     # scores of magnitude 2^7 carry 2^-17 of it as fp32 rounding of the scaled product, on top of the 2e-3 of the other tests
     assert np.abs(lse[0].cpu().numpy() - lo).max() < 2e-3 + np.abs(lo).max() * 2.0 ** -17
+
+
+@pytest.mark.parametrize("n,Hq,seg_bounds", [(2048, 2, [0, 2048]), (2112, 1, [0, 64, 2112]), (4160, 4, [0, 4160])])
+@pytest.mark.parametrize("out", [torch.float32, torch.bfloat16])
+def test_tiles_shared_by_a_cluster_match_the_oracle(n, Hq, seg_bounds, out):
+    """Launches of few tiles give a tile to 2, 4 or 8 CTAs.  Every pattern on one head, among them tiles with fewer chunks
+    than CTAs (block-sparse with one block, a window of one key), a segment of one block, a last tile of 64 rows."""
+    L = make_layer(tiny_spec(29 + n, n, Hq, 1))
+    p = rs.Problem(Hq, 1, n, seg_bounds)
+    Qs, Ks, Vs = f64_heads(L)
+    probes = oracle_probe_all(Qs, Ks, p)
+    lib = c_library(CANDS)
+    Q, K, V = dev_bf16(L["Q"]), dev_bf16(L["K"]), dev_bf16(L["V"])
+    for c in range(0, len(CANDS), Hq):
+        choice = [(c + item) % len(CANDS) for item in range(p.n_items)]
+        sets = oracle_index_sets(p, CANDS, choice, probes)
+        idx = upload_materialised(p, lib, sets)
+        O = torch.full((Hq, n, 128), float("nan"), dtype=out, device="cuda")
+        lse, onorm = torch.zeros((Hq, n), device="cuda"), torch.zeros((Hq, n), device="cuda")
+        st, counters = rs.new_status(), torch.zeros(2, dtype=torch.int64, device="cuda")
+        rs.rs_sparse_prefill_attn(p, Q, K, V, lib, idx, torch.tensor(choice, dtype=torch.int32, device="cuda"), O, lse, onorm,
+                                  counters, rs.new_workspace(p, lib), st)
+        rs.check_status(st, "shared tiles")
+        assert int(counters[1]) == Hq * sum((b - a + 127) // 128 for a, b in zip(seg_bounds[:-1], seg_bounds[1:]))
+        for item, ix in enumerate(sets):
+            h = item % Hq
+            rows = np.unique(np.concatenate([np.arange(ix.q0, min(ix.q0 + 130, ix.q1)), np.arange(max(ix.q0, ix.q1 - 130), ix.q1)]))
+            Oo, lo, no = A.masked_attention(Qs[h], Ks[0], Vs[0], lambda r, nk: PT.mask_rows(ix, r, nk), rows)
+            if out == torch.float32:
+                assert_attention_close(O[h, rows].cpu().numpy(), Oo, f"item {item} {ix.cand}")
+            else:                                  # rounded once more: 2^-9 of the value on top
+                assert np.abs(O[h, rows].float().cpu().numpy() - Oo).max() <= 2e-2 + np.abs(Oo).max() * 2.0 ** -9
+            assert np.abs(lse[h, rows].cpu().numpy() - lo).max() < 2e-3, ix.cand
+            assert np.all(np.abs(onorm[h, rows].cpu().numpy() - no) < 1e-2 * no + 1e-3)
