@@ -41,7 +41,7 @@ struct AttnParams {
   const int2* order;          // [n_work] (item, tile in segment), heavy first
   int split;                  // CTAs that share a tile's chunks (a cluster; 1: none)
   void* O;
-  int o_f32;
+  int o_f32, o_wide;          // fp32 output; output 32-byte aligned
   float* lse;
   float* onorm;
   unsigned long long* counters;
@@ -52,14 +52,6 @@ struct AttnParams {
 struct SmemLayout {   // offsets from the 1024-aligned base
   static constexpr uint32_t q = 0, k = 32768, v = 65536, end_tiles = 98304;
 };
-
-__device__ __forceinline__ uint32_t range_mask(int lo, int hi, int w) {
-  int a = max(lo, 32 * w), b = min(hi, 32 * w + 31);
-  if (a > b) return 0u;
-  uint32_t len = (uint32_t)(b - a + 1);
-  uint32_t m = (len == 32u) ? 0xffffffffu : ((1u << len) - 1u);
-  return m << (a - 32 * w);
-}
 
 // Masks one 64-key chunk of a score row in place in TMEM (rare chunks only: the causal diagonal, A-shape edges,
 // chunks another quarter wants, gathered vertical columns).  Kept out of line so that the common, unmasked chunk
@@ -221,6 +213,17 @@ __device__ __noinline__ float3 rs_raise_and_exp(uint32_t t_x, float sl2, float m
   return make_float3(m_run, l_run, sum);
 }
 
+// 32 bytes of one row: one store where the output is 32-byte aligned, two otherwise.
+__device__ __forceinline__ void store32(void* dst, const uint32_t (&w)[8], int wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+  } else {
+    reinterpret_cast<uint4*>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 // ------------------------------------------------------------------------------------------ tiles shared by a cluster
 // When a launch has too few tiles for the chip, `split` CTAs of a cluster take every split-th chunk of a tile and each ends
 // with its own (m, l, O).  Rank q owns rows [q 128 / split, ...): the rows' partial results travel to it through
@@ -368,7 +371,6 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tmem_alloc(smem_u32((const void*)&misc[0]), kTmemCols);
     tmem_relinquish();
   }
-  for (int i = tid; i < 128; i += kThreads) { lo_bits[i] = 0; hi_bits[i] = 0; d_bits[i] = 0; }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -399,143 +401,148 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     tma_load_2d(base + SmemLayout::q + 16384, &tmQ, bar_q, 64, h * P.n + i0);
   }
 
-  // ---- chunk list: bitmaps of key blocks wanted by the low / high 64 query rows, then ordered compaction
-  int vs_slot = 0, n_vcols = 0;
-  if (pattern == RS_VERTICAL_SLASH) {
-    vs_slot = P.vs_eval_layout ? item * P.n_cand + P.choice[item] : item;
-    const int* cnt = P.idx.vs_count + 4 * vs_slot;
-    n_vcols = cnt[0];
-    const int n_diag = cnt[2];
-    const int* dl = P.idx.vs_diag + (size_t)vs_slot * P.idx.nd_cap;
-    for (int i = tid; i < n_diag; i += kThreads) {
-      int dlt = dl[i];
-      if (dlt >= 0 && dlt < 4096) atomicOr(&d_bits[dlt >> 5], 1u << (dlt & 31));
-    }
-  } else if (pattern == RS_BLOCK_SPARSE) {
-    for (int half = 0; half < (has_hi ? 2 : 1); ++half) {
-      const size_t row = (size_t)h * (P.n >> 6) + qb0 + half;
-      const int cnt = P.idx.bs_count[row];
-      const int* bl = P.idx.bs_blk + row * P.idx.kb_cap;
-      uint32_t* dst = half ? hi_bits : lo_bits;
-      for (int i = tid; i < cnt; i += kThreads) {
-        int kb = bl[i];
-        if (kb >= 0 && kb <= qb0 + half) atomicOr(&dst[kb >> 5], 1u << (kb & 31));
+  // ---- the tile's chunks.  Dense and A-shape tiles visit [0, n_first) and [second, qb_last], which needs no list: building
+  // one takes seven block barriers, 2 to 4 us of the 16 a short tile costs beside its chunks.  The other patterns build one:
+  // bitmaps of key blocks wanted by the low / high 64 query rows, then ordered compaction.
+  int vs_slot = 0, n_vcols = 0, n_vis = 0, n_block;
+  const bool listed = pattern == RS_VERTICAL_SLASH || pattern == RS_BLOCK_SPARSE;
+  const int sink_blocks = pattern == RS_DENSE ? qb_last + 1 : cand.b0 > 0 ? ((cand.b0 - 1) >> 6) + 1 : 0;
+  const int win_lo = max(0, i0 - cand.b1 + 1) >> 6, win_hi = max(0, i0 + 64 - cand.b1 + 1) >> 6;
+  const int n_first = min(sink_blocks, qb_last + 1), second = max(win_lo, n_first);
+  auto entry = [&](int c) -> uint32_t {        // key block and flags of chunk c
+    if (listed) return list[c];
+    const int kb = c < n_first ? c : second + (c - n_first);
+    uint32_t e = (uint32_t)kb;
+    if (kb <= qb0 && (kb < sink_blocks || kb >= win_lo)) e |= F_LO;
+    if (has_hi && (kb < sink_blocks || kb >= win_hi)) e |= F_HI;
+    if (kb >= qb0) e |= F_CAUSAL;
+    if (pattern == RS_A_SHAPE && kb * 64 < i0 + kTileM - cand.b1 && (kb + 1) * 64 > cand.b0) e |= F_EDGE;
+    return e;
+  };
+  if (!listed) {
+    n_block = n_first + max(0, qb_last + 1 - second);
+  } else {
+    for (int i = tid; i < 128; i += kThreads) { lo_bits[i] = 0; hi_bits[i] = 0; d_bits[i] = 0; }
+    __syncthreads();
+    if (pattern == RS_VERTICAL_SLASH) {
+      vs_slot = P.vs_eval_layout ? item * P.n_cand + P.choice[item] : item;
+      const int* cnt = P.idx.vs_count + 4 * vs_slot;
+      n_vcols = cnt[0];
+      const int n_diag = cnt[2];
+      const int* dl = P.idx.vs_diag + (size_t)vs_slot * P.idx.nd_cap;
+      for (int i = tid; i < n_diag; i += kThreads) {
+        int dlt = dl[i];
+        if (dlt >= 0 && dlt < 4096) atomicOr(&d_bits[dlt >> 5], 1u << (dlt & 31));
+      }
+    } else if (pattern == RS_BLOCK_SPARSE) {
+      for (int half = 0; half < (has_hi ? 2 : 1); ++half) {
+        const size_t row = (size_t)h * (P.n >> 6) + qb0 + half;
+        const int cnt = P.idx.bs_count[row];
+        const int* bl = P.idx.bs_blk + row * P.idx.kb_cap;
+        uint32_t* dst = half ? hi_bits : lo_bits;
+        for (int i = tid; i < cnt; i += kThreads) {
+          int kb = bl[i];
+          if (kb >= 0 && kb <= qb0 + half) atomicOr(&dst[kb >> 5], 1u << (kb & 31));
+        }
       }
     }
-  }
-  __syncthreads();
-  if (pattern != RS_BLOCK_SPARSE) {
-    for (int wd = tid; wd < nb_words; wd += kThreads) {
-      uint32_t lo = 0, hi = 0;
-      if (pattern == RS_DENSE) {
-        lo = range_mask(0, qb0, wd);
-        hi = range_mask(0, qb0 + 1, wd);
-      } else if (pattern == RS_A_SHAPE) {
-        const int n_sink = cand.b0, win = cand.b1;
-        const uint32_t sink0 = (n_sink > 0) ? range_mask(0, min(qb0, (n_sink - 1) >> 6), wd) : 0u;
-        const uint32_t sink1 = (n_sink > 0) ? range_mask(0, min(qb0 + 1, (n_sink - 1) >> 6), wd) : 0u;
-        lo = sink0 | range_mask(max(0, i0 - win + 1) >> 6, qb0, wd);
-        hi = sink1 | range_mask(max(0, i0 + 64 - win + 1) >> 6, qb0 + 1, wd);
-      } else {   // vertical-slash: block kb is wanted by query block qb when (qb - kb) is in D
-        // bit b of the word stands for kb = 32 wd + b, i.e. for the diagonal qb - 32 wd - b: the word is a 32-bit
-        // window of D, read backwards
+    __syncthreads();
+    if (pattern == RS_VERTICAL_SLASH) {
+      for (int wd = tid; wd < nb_words; wd += kThreads) {
+        // vertical-slash: block kb is wanted by query block qb when (qb - kb) is in D.  Bit b of the word stands for
+        // kb = 32 wd + b, i.e. for the diagonal qb - 32 wd - b: the word is a 32-bit window of D, read backwards
         auto d_window = [&](int pos) -> uint32_t {      // D[pos .. pos + 31]; diagonals outside [0, 4096) are not in D
           const int w0 = pos >> 5;                      // arithmetic shift: floor
           const uint32_t a = (w0 >= 0 && w0 < 128) ? d_bits[w0] : 0u;
           const uint32_t b = (w0 + 1 >= 0 && w0 + 1 < 128) ? d_bits[w0 + 1] : 0u;
           return __funnelshift_r(a, b, (uint32_t)(pos & 31));
         };
-        lo = __brev(d_window(qb0 - 32 * wd - 31));
-        hi = __brev(d_window(qb0 + 1 - 32 * wd - 31));
+        lo_bits[wd] = __brev(d_window(qb0 - 32 * wd - 31));
+        hi_bits[wd] = has_hi ? __brev(d_window(qb0 + 1 - 32 * wd - 31)) : 0u;
       }
-      lo_bits[wd] = lo;
-      hi_bits[wd] = has_hi ? hi : 0u;
     }
-  }
-  __syncthreads();
-  if (warp == 0) {
-    // exclusive prefix of the words' chunk counts: a warp scan, 32 words at a time
-    int carry = 0;
-    for (int wbase = 0; wbase < nb_words; wbase += 32) {
-      const int wd = wbase + lane;
-      const int c = wd < nb_words ? __popc(lo_bits[wd] | hi_bits[wd]) : 0;
-      int incl = c;
+    __syncthreads();
+    if (warp == 0) {
+      // exclusive prefix of the words' chunk counts: a warp scan, 32 words at a time
+      int carry = 0;
+      for (int wbase = 0; wbase < nb_words; wbase += 32) {
+        const int wd = wbase + lane;
+        const int c = wd < nb_words ? __popc(lo_bits[wd] | hi_bits[wd]) : 0;
+        int incl = c;
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += t;
-      }
-      if (wd < nb_words) wprefix[wd] = carry + incl - c;
-      carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) misc[2] = carry;
-  } else if (pattern == RS_VERTICAL_SLASH && n_vcols > 0) {
-    // The other five warps walk the ascending list of gathered columns, 32 at a time.  Columns with j <= last valid
-    // row are a prefix: they are counted.  Per 32-column piece and row half: which columns survive for every row of
-    // the half (valid entry, key block not after the half's block, not already covered by a block diagonal of D) and
-    // which of them lie in the half's own key block; a chunk whose 64 columns all survive outside the own block needs
-    // no mask at all.
-    const int* vc = P.idx.vs_cols + (size_t)vs_slot * P.idx.kv_cap;
-    const int i_last = i0 + rows_valid - 1;
-    const int n_piece = (n_vcols + 31) >> 5;
-    int cnt = 0;
-    for (int piece = warp - 1; piece < n_piece; piece += kThreads / 32 - 1) {
-      const int vi = piece * 32 + lane;
-      const bool valid = vi < n_vcols;
-      const int j = valid ? vc[vi] : 0;
-      cnt += (valid && j <= i_last) ? 1 : 0;
-      if (piece < 2 * kMaskChunks) {
-        uint32_t kp[2], dg[2];
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const int dlt = qb0 + hf - (j >> 6);
-          const bool covered = dlt >= 0 && dlt < 4096 && ((d_bits[dlt >> 5] >> (dlt & 31)) & 1u);
-          const bool keep = valid && dlt >= 0 && !covered;
-          kp[hf] = __ballot_sync(0xffffffffu, keep);
-          dg[hf] = __ballot_sync(0xffffffffu, keep && dlt == 0);
+        for (int off = 1; off < 32; off <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, incl, off);
+          if (lane >= off) incl += t;
         }
-        if (lane == 0) {
-          uint32_t* k32 = reinterpret_cast<uint32_t*>(vkeep);
-          uint32_t* d32 = reinterpret_cast<uint32_t*>(vdiag);
-          const int chunk = piece >> 1, part = piece & 1;
-          k32[(chunk * 2 + 0) * 2 + part] = kp[0]; k32[(chunk * 2 + 1) * 2 + part] = kp[1];
-          d32[(chunk * 2 + 0) * 2 + part] = dg[0]; d32[(chunk * 2 + 1) * 2 + part] = dg[1];
+        if (wd < nb_words) wprefix[wd] = carry + incl - c;
+        carry += __shfl_sync(0xffffffffu, incl, 31);
+      }
+      if (lane == 0) misc[2] = carry;
+    } else if (pattern == RS_VERTICAL_SLASH && n_vcols > 0) {
+      // The other five warps walk the ascending list of gathered columns, 32 at a time.  Columns with j <= last valid
+      // row are a prefix: they are counted.  Per 32-column piece and row half: which columns survive for every row of
+      // the half (valid entry, key block not after the half's block, not already covered by a block diagonal of D) and
+      // which of them lie in the half's own key block; a chunk whose 64 columns all survive outside the own block needs
+      // no mask at all.
+      const int* vc = P.idx.vs_cols + (size_t)vs_slot * P.idx.kv_cap;
+      const int i_last = i0 + rows_valid - 1;
+      const int n_piece = (n_vcols + 31) >> 5;
+      int cnt = 0;
+      for (int piece = warp - 1; piece < n_piece; piece += kThreads / 32 - 1) {
+        const int vi = piece * 32 + lane;
+        const bool valid = vi < n_vcols;
+        const int j = valid ? vc[vi] : 0;
+        cnt += (valid && j <= i_last) ? 1 : 0;
+        if (piece < 2 * kMaskChunks) {
+          uint32_t kp[2], dg[2];
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int dlt = qb0 + hf - (j >> 6);
+            const bool covered = dlt >= 0 && dlt < 4096 && ((d_bits[dlt >> 5] >> (dlt & 31)) & 1u);
+            const bool keep = valid && dlt >= 0 && !covered;
+            kp[hf] = __ballot_sync(0xffffffffu, keep);
+            dg[hf] = __ballot_sync(0xffffffffu, keep && dlt == 0);
+          }
+          if (lane == 0) {
+            uint32_t* k32 = reinterpret_cast<uint32_t*>(vkeep);
+            uint32_t* d32 = reinterpret_cast<uint32_t*>(vdiag);
+            const int chunk = piece >> 1, part = piece & 1;
+            k32[(chunk * 2 + 0) * 2 + part] = kp[0]; k32[(chunk * 2 + 1) * 2 + part] = kp[1];
+            d32[(chunk * 2 + 0) * 2 + part] = dg[0]; d32[(chunk * 2 + 1) * 2 + part] = dg[1];
+          }
         }
       }
-    }
-    // an odd number of pieces: the second half of the last chunk holds no column
-    if (warp == 1 && lane == 0 && (n_piece & 1) && n_piece < 2 * kMaskChunks) {
-      uint32_t* k32 = reinterpret_cast<uint32_t*>(vkeep);
-      uint32_t* d32 = reinterpret_cast<uint32_t*>(vdiag);
-      const int chunk = n_piece >> 1;
-      k32[(chunk * 2 + 0) * 2 + 1] = 0u; k32[(chunk * 2 + 1) * 2 + 1] = 0u;
-      d32[(chunk * 2 + 0) * 2 + 1] = 0u; d32[(chunk * 2 + 1) * 2 + 1] = 0u;
-    }
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (lane == 0 && cnt > 0) atomicAdd(const_cast<int*>(&misc[3]), cnt);
-  }
-  __syncthreads();
-  for (int wd = tid; wd < nb_words; wd += kThreads) {
-    uint32_t lo = lo_bits[wd], hi = hi_bits[wd], any = lo | hi;
-    int at = wprefix[wd];
-    while (any) {
-      const int b = __ffs(any) - 1;
-      any &= any - 1;
-      const int kb = 32 * wd + b;
-      uint32_t e = (uint32_t)kb;
-      if ((lo >> b) & 1u) e |= F_LO;
-      if ((hi >> b) & 1u) e |= F_HI;
-      if (kb >= qb0) e |= F_CAUSAL;
-      if (pattern == RS_A_SHAPE) {
-        const bool in_window = kb * 64 >= i0 + kTileM - cand.b1;
-        const bool in_sink = (kb + 1) * 64 <= cand.b0;
-        if (!in_window && !in_sink) e |= F_EDGE;
+      // an odd number of pieces: the second half of the last chunk holds no column
+      if (warp == 1 && lane == 0 && (n_piece & 1) && n_piece < 2 * kMaskChunks) {
+        uint32_t* k32 = reinterpret_cast<uint32_t*>(vkeep);
+        uint32_t* d32 = reinterpret_cast<uint32_t*>(vdiag);
+        const int chunk = n_piece >> 1;
+        k32[(chunk * 2 + 0) * 2 + 1] = 0u; k32[(chunk * 2 + 1) * 2 + 1] = 0u;
+        d32[(chunk * 2 + 0) * 2 + 1] = 0u; d32[(chunk * 2 + 1) * 2 + 1] = 0u;
       }
-      list[at++] = (uint16_t)e;
+      cnt = __reduce_add_sync(0xffffffffu, cnt);
+      if (lane == 0 && cnt > 0) atomicAdd(const_cast<int*>(&misc[3]), cnt);
     }
+    __syncthreads();
+    for (int wd = tid; wd < nb_words; wd += kThreads) {
+      uint32_t lo = lo_bits[wd], hi = hi_bits[wd], any = lo | hi;
+      int at = wprefix[wd];
+      while (any) {
+        const int b = __ffs(any) - 1;
+        any &= any - 1;
+        const int kb = 32 * wd + b;
+        uint32_t e = (uint32_t)kb;
+        if ((lo >> b) & 1u) e |= F_LO;
+        if ((hi >> b) & 1u) e |= F_HI;
+        if (kb >= qb0) e |= F_CAUSAL;
+        list[at++] = (uint16_t)e;
+      }
+    }
+    __syncthreads();
+    n_block = warp_uniform(misc[2]);
+    n_vis = warp_uniform(misc[3]);             // visible gathered columns
   }
-  __syncthreads();
-  const int n_block = warp_uniform(misc[2]), n_vert = (warp_uniform(misc[3]) + kChunk - 1) / kChunk;     // misc[3]: visible gathered columns
+  const int n_vert = (n_vis + kChunk - 1) / kChunk;
   const int n_chunks = (n_block + n_vert - rank + split - 1) / split;
   float m_run = -INFINITY, l_run = 0.f;      // softmax threads: reference and sum of their row
   // =========================================================================================== roles
@@ -550,7 +557,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       auto load_chunk = [&](int ch, uint32_t dst, uint32_t bar, const CUtensorMap* tm_blocks, const CUtensorMap* tm_packed) {
         mbar_arrive_expect_tx(bar, 16384u);
         if (ch < n_block) {
-          const int row = g * P.n + (int)(list[ch] & 0xfffu) * kChunk;
+          const int row = g * P.n + (int)(entry(ch) & 0xfffu) * kChunk;
           tma_load_2d(dst, tm_blocks, bar, 0, row);
           tma_load_2d(dst + 16384, tm_blocks, bar, 64, row);
         } else {
@@ -665,7 +672,7 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         unsigned long long vk = 0ull, vd = 0ull;
         const int gch = rank + split * ch;
         if (gch < n_block) {
-          const uint32_t e = list[gch];
+          const uint32_t e = entry(gch);
           if (!(e & (half ? F_HI : F_LO))) {
             mode = 0;
           } else if (e & (F_CAUSAL | F_EDGE)) {
@@ -744,17 +751,27 @@ rs_attn_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         float f[32];
 #pragma unroll
         for (int x = 0; x < 32; ++x) { f[x] = __uint_as_float(v[x]) * inv; ss = fmaf(f[x], f[x], ss); }
+        // A thread owns a row, so a warp's store touches 32 lines whatever its width: the fewer instructions the better
+        // (32 bytes a thread where O is aligned to that).
         if (valid) {
           if (P.o_f32) {
-            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float*>(P.O) + orow + c4 * 32);
+            float* dst = reinterpret_cast<float*>(P.O) + orow + c4 * 32;
 #pragma unroll
-            for (int x = 0; x < 8; ++x) dst[x] = make_float4(f[4 * x], f[4 * x + 1], f[4 * x + 2], f[4 * x + 3]);
+            for (int x = 0; x < 4; ++x) {
+              uint32_t w8[8];
+#pragma unroll
+              for (int y = 0; y < 8; ++y) w8[y] = __float_as_uint(f[8 * x + y]);
+              store32(dst + 8 * x, w8, P.o_wide);
+            }
           } else {
-            uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(P.O) + orow + c4 * 32);
+            __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(P.O) + orow + c4 * 32;
 #pragma unroll
-            for (int x = 0; x < 4; ++x)
-              dst[x] = make_uint4(pack_bf16x2(f[8 * x], f[8 * x + 1]), pack_bf16x2(f[8 * x + 2], f[8 * x + 3]),
-                                  pack_bf16x2(f[8 * x + 4], f[8 * x + 5]), pack_bf16x2(f[8 * x + 6], f[8 * x + 7]));
+            for (int x = 0; x < 2; ++x) {
+              uint32_t w8[8];
+#pragma unroll
+              for (int y = 0; y < 8; ++y) w8[y] = pack_bf16x2(f[16 * x + 2 * y], f[16 * x + 2 * y + 1]);
+              store32(dst + 16 * x, w8, P.o_wide);
+            }
           }
         }
       }
@@ -950,7 +967,7 @@ int enqueue_attn(const rs_problem* p, const void* Q, const void* K, const void* 
   P.vs_eval_layout = vs_eval_layout ? 1 : 0;
   P.kv_pad = sc.kv_pad;
   P.order = sc.order;
-  P.O = O; P.o_f32 = o_dtype; P.lse = lse; P.onorm = onorm;
+  P.O = O; P.o_f32 = o_dtype; P.o_wide = ((uintptr_t)O & 31) == 0 ? 1 : 0; P.lse = lse; P.onorm = onorm;
   P.counters = reinterpret_cast<unsigned long long*>(counters);
   P.status = status;
   P.scale_log2e = (float)(1.4426950408889634 / sqrt((double)RS_HEAD_DIM));
